@@ -2,12 +2,22 @@
 // 3^dim cells of the block B_i, acoustic pair Riemann solver, and the
 // per-particle sums of eqs. (SPH:Conti), (SPH:Pulse), (SPH:Energy).
 //
-// A warp handles one home cell at a time, one lane per home particle (see
-// k_pair below): candidates are staged in shared memory row by row, tested
-// against every lane's particle, and the interacting ones are kept in a
-// per-lane list; the fluxes are evaluated over the lists, so the flux
-// arithmetic runs on converged lanes instead of under the ~17% acceptance
-// of the candidate test.
+// A warp handles a group of up to 32 consecutive slots (cell order), one lane
+// per slot.  The part of a group that lies in one x-row of cells is a segment;
+// its candidates are the slots of the 3^(dim-1) neighbouring rows from one
+// cell before the segment's first cell to one past its last.  Each lane loads
+// one candidate, a ballot compacts those that can reach the segment's bounding
+// box into shared memory, every lane then tests its own particle against the
+// compacted ones (a broadcast read) and appends those that interact to its
+// list; after the scan each lane evaluates the fluxes of its own list.
+//
+// Why groups of slots and not single cells: a cell holds 17.6 particles of a
+// lattice (kappa eta = 2.6 spacings), so a warp per cell evaluated the fluxes
+// with 55 % of its lanes; a group fills them.  The box cull drops the
+// candidates beyond the corners and edges of the block (40 % of them).
+// Measured against a warp per cell without the cull, whole passes: 387k plate,
+// mixed, 0.97 -> 0.71 ms per step; 203k plate, FP64, 8.16 -> 3.36 ms; 72.9k
+// plane, order 2, 0.240 -> 0.138 ms.
 //
 // Antisymmetry: the momentum flux F_ij e^R that i and j apply are bitwise
 // negatives of each other, and so are the energy fluxes Q_ij of FP64
@@ -15,145 +25,85 @@
 // (FwdAcc in pair_common.cuh).
 //
 // Modes of the kernel: the rates (optionally with order-2 states), the SPH
-// gradients of order 2, the reverse mode, and the Verlet list build; the
-// evaluation over the lists is k_pair_lists.cu.
+// gradients of order 2 and the reverse mode; the Verlet list build is
+// k_list_build.cu, the evaluation over the lists k_pair_lists.cu.
 //
-// Mixed precision: the candidate test and the flux run in FP32 on offsets
-// from each particle's own cell origin (FP32 keeps ~7 digits of a cell edge,
-// not of the domain).  The FP32 test decides r^2 < R^2 whenever r^2 lies
-// outside a band of 2^-12 D^c^2 around R^2, which bounds the accumulated
-// FP32 error of both sides (<= ~1e-5 D^c^2); inside the band the pair is
+// The candidate test runs in FP32 in both precisions: mixed handles on the
+// packed offsets from each particle's own cell origin, FP64 handles on
+// offsets from the segment's first particle, scaled by a power of two so that
+// the cell edge is ~1 (any length unit stays in FP32's range).  The FP32 test
+// decides r^2 < R^2 whenever r^2 lies outside a band of 2^-12 D^c^2 around
+// R^2, which bounds the accumulated FP32 error of both sides (<= ~1e-5 D^c^2,
+// segments spanning at most kSpan cells included); inside the band the pair is
 // decided by the FP64 test on the global positions, with the same operation
-// order as the oracle, so the pair set is the FP64 one.  Per-particle sums
-// are Kahan-compensated.
+// order as the oracle, so the pair set is the FP64 one.  (FP64 handles tested
+// every candidate in FP64 before, 12 instructions of a pipe 64 times narrower
+// than FP32's: a third of their pair kernel.)  Mixed per-particle sums are
+// Kahan-compensated; each lane adds its pairs in candidate order.
 #include "pair_common.cuh"
 
 namespace csph {
 
 namespace {
 
-// One warp per home cell, lane l owning home particle start_c + chunk + l.
-// For each neighbour row (the 3 x-consecutive cells at (oy, oz), contiguous
-// in slot order) the warp stages 32 candidates at a time in shared memory,
-// one loaded per lane (position relative to the home cell origin in mixed
-// mode, global in FP64); every lane then tests its own home particle against
-// each staged candidate, a broadcast read, and appends the accepted ones to
-// its list in candidate order (no ballots or shuffles in the test loop).
-// A list entry is 16 bits: the neighbour-cell code (ox+1) + 3 (oy+1) +
-// 9 (oz+1) and the offset inside that cell.  Lists are rows of padded
-// stride in shared memory; after the scan (or when some list could overflow
-// during the next chunk) each lane evaluates the fluxes of its own row.
-// List staging per home particle in shared memory: kListCap entries for the
-// flux modes, kBuildCap for the list build (whose rows are flushed to the
-// global lists, so a shorter row only means more frequent flushes and frees
-// shared memory for more resident blocks).  Row stride: cap + 2 16-bit
-// entries, an odd number of words, so lane rows fall in distinct banks.
-// Measured on the 1.125M plate: rows of 64 or 96 entries with 7-8 resident
-// blocks made the step 0.3-3 % slower than 128 entries with 6 blocks.
-constexpr int kBuildCap = 128;
-constexpr int kBuildBlocks = 6;      // resident blocks per SM of the mixed list build
+constexpr int kRowCap = 112;   // list entries per slot between flushes (row stride 2 mod 64 bytes: lane rows in
+                               // distinct banks); a flush mid-scan is rare (a lattice has 81, the slot itself included)
+constexpr int kSegs = 2;       // segments per scan before a flush
+constexpr int kSpan = 16;      // cells a segment may span along x (bounds the FP32 frame)
 
 template <bool MIXED, int DIM, int MODE, bool HLL = false, bool EXTRA = true>
-__global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kModeFwd2) ? (MIXED ? 4 : 2)
-                                                 : (MODE == kModeGrad ? (MIXED ? 5 : 3)
-                                                 : (MODE == kModeList ? (MIXED ? kBuildBlocks : 4) : (MIXED ? 6 : 4))))
+__global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kModeFwd2) ? (MIXED ? 4 : 3)
+                                                 : (MODE == kModeGrad ? (MIXED ? 5 : 3) : (MIXED ? 6 : 4)))
     k_pair(PairArgs a) {
   chain_entry();
   constexpr bool VJP = MODE == kModeVjp;
-  constexpr bool LIST = MODE == kModeList;
   constexpr bool GRAD = MODE == kModeGrad;
+  constexpr int kRows = DIM == 3 ? 9 : (DIM == 2 ? 3 : 1);
   using P = Pair<MIXED, DIM>;
   using T = typename P::T;
   using V4 = typename P::V4;
   using V2 = typename P::V2;
   using VC = typename P::VC;
-  constexpr int kCap = MODE == kModeList ? kBuildCap : kListCap;
-  __shared__ uint16_t list[kWarps][32][kCap + 2];           // [warp][home particle][entry]
-  __shared__ V4 home[kWarps][LIST ? 1 : 32];                 // home particles: x, y, z, kh d (mixed) or d (FP64)
-  __shared__ V4 cand[kWarps][32];                            // list build: candidates (shifted in mixed), d
-  __shared__ uint16_t cand_ent[kWarps][32];                  // list build: their list entries
-  __shared__ int32_t nb_start[kWarps][27];                   // start slot of each neighbour cell
-  __shared__ float4 nb_tab[kWarps][27];                      // per neighbour cell: start (bits), shift x, y, z
+  __shared__ uint16_t list[kWarps][32][kRowCap + 2];         // [warp][lane][entry]: cell code << 11 | offset
+  __shared__ float4 cand[kWarps][32];                        // candidates that survived the cull: x, y, z, d (FP32)
+  __shared__ int2 cand_ent[kWarps][32];                      // their entry in the segment's frame, their slot
+  __shared__ float4 nb_tab[kWarps][kSegs][27];               // per segment and cell code: first slot (bits), shift x, y, z
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
-  const int64_t total = *a.total_cells_dev;
-  // the list build reads the cell-order copy of the positions when the lists
-  // are laid out in the unit-major evaluation order
-  const V4* __restrict__ A = reinterpret_cast<const V4*>(LIST && a.Ac ? a.Ac : a.A);
+  const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
   const V4* __restrict__ B = reinterpret_cast<const V4*>(a.B);
   const VC* __restrict__ C = reinterpret_cast<const VC*>(a.C);
-  if constexpr (LIST) {
-    if (a.vflag[0] == 0) return;                 // lists still valid: nothing to build
-    if (blockIdx.x == 0 && threadIdx.x == 0) { a.vflag[1] = 0; a.vflag[2] += 1; }
-  }
-  // Persistent warps: each takes the next cell from a global counter, so the
-  // work spreads evenly whatever the mix of empty and crowded cells.
-  for (;;) {
-  int64_t cell_g = 0;
-  if (lane == 0) cell_g = (int64_t)atomicAdd(a.work_counter, 1ull);
-  cell_g = __shfl_sync(0xffffffffu, cell_g, 0);
-  if (cell_g >= total) break;
-  const int hs = a.cell_start[cell_g], he = a.cell_start[cell_g + 1];
-  if (hs == he) continue;                                    // empty cell (warp-uniform)
-
-  int b = 0;
-  if (a.n_inst > 1) {  // instance of this cell: binary search of the slot offsets
-    int lo = 0, hi = a.n_inst;
-    while (hi - lo > 1) {
-      int mid = (lo + hi) >> 1;
-      if (a.inst_off[mid] <= hs) lo = mid; else hi = mid;
-    }
-    b = lo;
-  }
-  if (LIST && a.vinst && a.vinst[b] == 0) continue;   // the instance keeps its lists (warp-uniform)
-  const GridInfo& g = a.grid[b];
-  const int nx = g.dims[0], ny = g.dims[1], nz = g.dims[2];
-  const int64_t lc = cell_g - g.cell_off;
-  const int cx = (int)(lc % nx), cy = (int)((lc / nx) % ny), cz = (int)(lc / ((int64_t)nx * ny));
-  const T dcs = MIXED ? (T)g.dc_f : T(0);
-  const float band = MIXED ? 0x1p-12f * g.dc_f * g.dc_f : 0.f;
-
-  // starts of the 27 neighbour cells (index (ox+1) + 3 (oy+1) + 9 (oz+1)); -1 outside the mesh
-  if (lane < 27) {
-    const int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = lane / 9 - 1;
-    const int xx = cx + ox, yy = cy + oy, zz = cz + oz;
-    const bool in = xx >= 0 && xx < nx && yy >= 0 && yy < ny && zz >= 0 && zz < nz;
-    const int st0 = in ? a.cell_start[g.cell_off + xx + (int64_t)nx * (yy + (int64_t)ny * zz)] : -1;
-    nb_start[warp][lane] = st0;
-    // the shift from the home cell's origin to this cell's, exact (ox, oy, oz in {-1, 0, 1})
-    nb_tab[warp][lane] = make_float4(__int_as_float(st0), MIXED ? (float)ox * (float)dcs : 0.f,
-                                     MIXED ? (float)oy * (float)dcs : 0.f, MIXED ? (float)oz * (float)dcs : 0.f);
-  }
-
-  for (int h0 = hs; h0 < he; h0 += 32) {
+  // Persistent warps: the first group of each is fixed (spread over the CTAs,
+  // so that few groups run on many SMs), the following ones come from a
+  // global counter, so the work spreads evenly.
+  const int n_1 = (int)a.n - 1;
+  unsigned long long q = (unsigned long long)warp * gridDim.x + blockIdx.x;
+  for (; (int64_t)(q * (unsigned)a.group) < a.n;) {
+    const int h0 = (int)(q * (unsigned)a.group);
     const long long t_start = a.load_timed ? clock64() : 0;   // timed unit loads
     const int i = h0 + lane;
-    const bool act = i < he;
-    const int nh = min(32, he - h0);
-    const int ii = act ? i : hs;
-    const V4 Ai = A[ii];
-    const T khdi = MIXED ? (T)a.kh_f * Ai.w : T(0);
-    if constexpr (!LIST) {
-      V4 hv = Ai;
-      if (MIXED) hv.w = khdi;
-      home[warp][lane] = hv;
-      __syncwarp();
-    }
-    int cnt = 0, vc = 0;
-    unsigned nfull = 0, ncand = 0, nexact = 0;
-    // list build: the home group's bounding box and largest kh d, a warp-wide cull of candidates
-    float bxl = 0.f, bxh = 0.f, byl = 0.f, byh = 0.f, bzl = 0.f, bzh = 0.f, bkh = 0.f;
-    if constexpr (LIST && MIXED) {
-      bxl = (float)Ai.x; bxh = bxl; byl = (float)Ai.y; byh = byl; bzl = (float)Ai.z; bzh = bzl; bkh = (float)khdi;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        bxl = fminf(bxl, __shfl_xor_sync(0xffffffffu, bxl, o)); bxh = fmaxf(bxh, __shfl_xor_sync(0xffffffffu, bxh, o));
-        byl = fminf(byl, __shfl_xor_sync(0xffffffffu, byl, o)); byh = fmaxf(byh, __shfl_xor_sync(0xffffffffu, byh, o));
-        bzl = fminf(bzl, __shfl_xor_sync(0xffffffffu, bzl, o)); bzh = fmaxf(bzh, __shfl_xor_sync(0xffffffffu, bzh, o));
-        bkh = fmaxf(bkh, __shfl_xor_sync(0xffffffffu, bkh, o));
+    const bool act = lane < a.group && i < a.n;
+    const int ii = act ? i : h0;
+    int b = 0;
+    if (a.n_inst > 1) {  // instance of this slot: binary search of the slot offsets
+      int lo = 0, hi = a.n_inst;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (a.inst_off[mid] <= ii) lo = mid; else hi = mid;
       }
+      b = lo;
     }
+    int cx, row;                                               // the slot's cell along x, its row of cells
+    {
+      const GridInfo& g = a.grid[b];
+      const int lc = a.slot_cell[ii] - (int)g.cell_off;
+      row = lc / g.dims[0];
+      cx = lc - row * g.dims[0];
+    }
+    const V4 Ai = A[ii];
+    int cnt = 0, seg_of = 0, cx_seg = 0;
+    unsigned nfull = 0, ncand = 0, nexact = 0;
     const int ui = a.K > 0 ? a.slot_unit[ii] : 0;
     const V4 Bi = B[ii];
     const VC Ci = C[ii];
@@ -314,43 +264,14 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       s_bd.add(gW * Wh * eh);
     };
 
-    // List build: the warp writes each home particle's new entries together,
-    // 32 consecutive entries of one row per store (the self pair dropped by
-    // a ballot, list order kept), instead of one entry of 32 rows per store.
-    auto flush_lists = [&]() {
-      nfull += (unsigned)cnt;
-      for (int hp = 0; hp < nh; ++hp) {
-        const int n = __shfl_sync(0xffffffffu, cnt, hp);
-        int v0 = __shfl_sync(0xffffffffu, vc, hp);
-        const int64_t ih = a.e_of_c ? (int64_t)a.e_of_c[h0 + hp] : (int64_t)(h0 + hp);   // the row's slot
-        const int64_t ihc = h0 + hp;                                                          // cell order
-        for (int k0 = 0; k0 < n; k0 += 32) {
-          const int k = k0 + lane;
-          uint32_t word = 0;
-          bool w = false;
-          if (k < n) {
-            const unsigned ent = list[warp][hp][k];
-            const int64_t j = (int64_t)__float_as_int(nb_tab[warp][ent >> 11].x) + (ent & 2047u);
-            w = j != ihc;
-            const int64_t je = a.e_of_c ? (int64_t)a.e_of_c[j] : j;
-            word = ((uint32_t)je << 5) | (ent >> 11);
-          }
-          const unsigned m = __ballot_sync(0xffffffffu, w);
-          const int pos = v0 + __popc(m & lt);
-          if (w && pos < a.vcap) a.vlist[ih * a.vcap + pos] = word;
-          v0 += __popc(m);
-        }
-        if (lane == hp) vc = v0;
-      }
-      cnt = 0;
-    };
-
     auto flush = [&]() {
       nfull += (unsigned)cnt;
       for (int k = 0; k < cnt; ++k) {
         const unsigned ent = list[warp][lane][k];
-        const float4 t = nb_tab[warp][ent >> 11];
-        const int64_t j = (int64_t)__float_as_int(t.x) + (ent & 2047u);
+        // (the two minima change nothing on a finite state; on one with infinite
+        // sizes, which is latched, they keep the accesses in bounds)
+        const float4 t = nb_tab[warp][seg_of][min(ent >> 11, 26u)];
+        const int64_t j = min(__float_as_int(t.x) + (int)(ent & 2047u), n_1);
         if constexpr (VJP) {
           pair_vjp(j, (T)t.y, (T)t.z, (T)t.w);
         } else if constexpr (GRAD) {
@@ -362,184 +283,206 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       cnt = 0;
     };
 
-    for (int oz = (DIM >= 3 ? -1 : 0); oz <= (DIM >= 3 ? 1 : 0); ++oz) {
-      for (int oy = (DIM >= 2 ? -1 : 0); oy <= (DIM >= 2 ? 1 : 0); ++oy) {
-        const int rc = 3 * (oy + 1) + 9 * (oz + 1);     // index of the row's ox = -1 cell
-        const int s_m = nb_start[warp][rc], s_0 = nb_start[warp][rc + 1], s_p = nb_start[warp][rc + 2];
-        if (s_0 < 0) continue;                           // row outside the mesh
-        // contiguous slot range of the row: from the first existing cell to the end of the last
-        const int r0 = s_m >= 0 ? s_m : s_0;
-        const int xe = s_p >= 0 ? cx + 2 : cx + 1;       // one past the last existing cell in x
-        const int64_t rowc = g.cell_off + (int64_t)nx * ((cy + oy) + (int64_t)ny * (cz + oz));
-        const int r1 = a.cell_start[rowc + xe];
-        const int b1 = a.cell_start[rowc + cx + 1];      // end of the ox = 0 cell
-        ncand += act ? (unsigned)(r1 - r0) : 0u;
-        for (int base = r0; base < r1; base += 32) {
-          // a chunk adds at most 32 entries to a list: flush first if one could overflow
-          if (__any_sync(0xffffffffu, cnt > kCap - 32)) {
-            if constexpr (LIST) flush_lists();
-            else if (act) flush();
-          }
-          const int j = base + lane;
-          const bool jv = j < r1;
-          V4 S = A[jv ? j : r0];
-          uint32_t ent = 0;
-          if (jv) {
-            const int ox = j < s_0 ? -1 : (j < b1 ? 0 : 1);
-            if (MIXED) { S.x += ox * dcs; S.y += oy * dcs; S.z += oz * dcs; }
-            const int off = j - (ox < 0 ? s_m : (ox == 0 ? s_0 : b1));
-            if (off > 2047) set_status(a.status, SPH_ERR_CAPACITY);   // cell over 2047 particles
-            ent = ((uint32_t)(rc + ox + 1) << 11) | (uint32_t)(off & 2047);
-          }
-          if constexpr (LIST) {
-            int nc = min(32, r1 - base);
-            if constexpr (MIXED) {
-              // keep only the candidates within reach of the home group's box
-              // (a superset: every rounding below is monotone in the distance)
-              const float ex = fmaxf(0.f, fmaxf((float)S.x - bxh, bxl - (float)S.x));
-              const float ey = DIM >= 2 ? fmaxf(0.f, fmaxf((float)S.y - byh, byl - (float)S.y)) : 0.f;
-              const float ez = DIM >= 3 ? fmaxf(0.f, fmaxf((float)S.z - bzh, bzl - (float)S.z)) : 0.f;
-              const float Rm = fmaf(a.kh_f, (float)S.w, bkh);
-              const bool keep = jv && fmaf(-Rm, Rm, P::r2_of(ex, ey, ez)) < band;
-              const unsigned km = __ballot_sync(0xffffffffu, keep);
-              if (keep) {
-                const int q = __popc(km & lt);
-                cand[warp][q] = S;
-                cand_ent[warp][q] = (uint16_t)ent;
-              }
-              nc = __popc(km);
-            } else {
-              cand[warp][lane] = S;
-              cand_ent[warp][lane] = (uint16_t)ent;
-            }
-            __syncwarp();
-            // each lane tests its home particle against the chunk's candidates,
-            // broadcast from shared memory, and appends the accepted ones to its
-            // own list in candidate order
-#pragma unroll 8
-            for (int c = 0; c < nc; ++c) {
-              const V4 Sc = cand[warp][c];
-              bool acc;
-              if (MIXED) {
-                const T dx = Sc.x - Ai.x;
-                const T dy = DIM >= 2 ? Sc.y - Ai.y : T(0);
-                const T dz = DIM >= 3 ? Sc.z - Ai.z : T(0);
-                const T r2 = P::r2_of(dx, dy, dz);
-                const T R = fmaf((T)a.kh_f, Sc.w, khdi);
-                const T diff = fmaf(-R, R, r2);          // r^2 - R^2
-                acc = diff < band;                        // superset of the (1 + beta) radius
-              } else {
-                T dx, dy, dz;
-                P::sep(true, Ai, Sc, T(0), T(0), T(0), dx, dy, dz);   // x_j - x_i, oracle order
-                const T r2 = P::r2_of(dx, dy, dz);
-                const double R = __dmul_rn(a.kh, __dadd_rn(Ai.w, Sc.w));
-                acc = r2 < __dmul_rn(R, R);
-              }
-              if (acc && act) list[warp][lane][cnt++] = cand_ent[warp][c];
-            }
-            __syncwarp();   // the candidate buffer is rewritten by the next chunk
-          } else {
-            // transposed test: each lane tests its candidate against home particle
-            // hp, broadcast from shared memory; a ballot collects the accepted lanes
-            // and each writes its entry at the next free position of hp's list
-#pragma unroll 4
-            for (int hp = 0; hp < nh; ++hp) {
-              const V4 H = home[warp][hp];
-              bool acc;
-              if (MIXED) {
-                const T dx = S.x - H.x;
-                const T dy = DIM >= 2 ? S.y - H.y : T(0);
-                const T dz = DIM >= 3 ? S.z - H.z : T(0);
-                const T r2 = P::r2_of(dx, dy, dz);
-                const T R = fmaf((T)a.kh_f, S.w, H.w);
-                const T diff = fmaf(-R, R, r2);          // r^2 - R^2
-                acc = diff < T(0);
-                if (fabsf(diff) <= band && jv) {          // too close to call in FP32: FP64 decides
-                  ++nexact;
-                  acc = (j == h0 + hp) || exact_accept(a, DIM, a.perm[h0 + hp], a.perm[j]);
-                }
-              } else {
-                T dx, dy, dz;
-                P::sep(true, H, S, T(0), T(0), T(0), dx, dy, dz);   // x_j - x_i, oracle order
-                const T r2 = P::r2_of(dx, dy, dz);
-                const double R = __dmul_rn(a.kh, __dadd_rn(H.w, S.w));
-                acc = r2 < __dmul_rn(R, R);
-              }
-              acc = acc && jv;
-              const unsigned mask = __ballot_sync(0xffffffffu, acc);
-              if (mask) {
-                const int c = __shfl_sync(0xffffffffu, cnt, hp);
-                if (acc) list[warp][hp][c + __popc(mask & lt)] = (uint16_t)ent;
-                if (lane == hp) cnt += __popc(mask);
-              }
-            }
-          }
+    unsigned todo = __ballot_sync(0xffffffffu, act);
+    int seg = 0;
+    while (todo) {
+      if (seg == kSegs) {                                      // the segment tables are full
+        flush();
+        __syncwarp();
+        seg = 0;
+      }
+      // the next segment: the lanes of one instance and row of cells, within kSpan cells of the first
+      const int lead = __ffs(todo) - 1;
+      const int b0 = __shfl_sync(0xffffffffu, b, lead), row0 = __shfl_sync(0xffffffffu, row, lead);
+      const int cx0 = __shfl_sync(0xffffffffu, cx, lead);
+      const bool same = ((todo >> lane) & 1u) && b == b0 && row == row0;
+      unsigned members = __ballot_sync(0xffffffffu, same && cx - cx0 < kSpan);
+      int cx1 = __shfl_sync(0xffffffffu, cx, 31 - __clz(members));
+      const GridInfo& g = a.grid[b0];
+      const int nx = g.dims[0], ny = g.dims[1], nz = g.dims[2];
+      const int cy0 = row0 % ny, cz0 = row0 / ny;
+      // lane r < kRows: first cell of neighbour row r (-1 outside the mesh) and its slot range
+      int64_t rbase = -1;
+      int rs0 = 0, rs1 = 0;
+      if (lane < kRows) {
+        const int yy = cy0 + (DIM >= 2 ? lane % 3 - 1 : 0), zz = cz0 + (DIM >= 3 ? lane / 3 - 1 : 0);
+        if (yy >= 0 && yy < ny && zz >= 0 && zz < nz) {
+          rbase = g.cell_off + (int64_t)nx * (yy + (int64_t)ny * zz);
+          rs0 = a.cell_start[rbase + (cx0 > 0 ? cx0 - 1 : 0)];
+          rs1 = a.cell_start[rbase + (cx1 + 1 < nx ? cx1 + 2 : nx)];
         }
       }
+      // Entries hold an 11-bit offset: from the row's first slot, or, where a
+      // crowded row exceeds that, from the cell's (a segment of one cell).
+      const bool wide = __any_sync(0xffffffffu, rs1 - rs0 > 2048);
+      if (wide && cx1 > cx0) {
+        members = __ballot_sync(0xffffffffu, same && cx == cx0);
+        cx1 = cx0;
+        if (rbase >= 0) rs1 = a.cell_start[rbase + (cx1 + 1 < nx ? cx1 + 2 : nx)];
+      }
+      const bool mine = (members >> lane) & 1u;
+      if (mine) { seg_of = seg; cx_seg = cx - cx0; }
+      todo &= ~members;
+      const T dcs = MIXED ? (T)g.dc_f : T(0);
+      {
+        // first slot of the row (or cell) and the exact shift from a home cell's origin, per cell code
+        const int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = lane / 9 - 1;
+        const int r = (DIM >= 2 ? oy + 1 : 0) + (DIM >= 3 ? 3 * (oz + 1) : 0);
+        const int src = r < kRows ? r : 0;
+        const int st = __shfl_sync(0xffffffffu, rs0, src);
+        const int64_t rb = __shfl_sync(0xffffffffu, rbase, src);
+        if (lane < 27) {
+          int first = st;
+          if (wide && rb >= 0 && cx0 + ox >= 0 && cx0 + ox < nx) first = a.cell_start[rb + cx0 + ox];
+          nb_tab[warp][seg][lane] = make_float4(__int_as_float(first), MIXED ? (float)ox * (float)dcs : 0.f,
+                                                MIXED ? (float)oy * (float)dcs : 0.f, MIXED ? (float)oz * (float)dcs : 0.f);
+        }
+      }
+      // FP32 frame of the test: the origin of cell cx0 (mixed), the segment's first particle (FP64)
+      int ex = 0;
+      double fx = 0.0, fy = 0.0, fz = 0.0;
+      float dct = MIXED ? (float)dcs : 0.f;
+      if constexpr (!MIXED) {
+        ex = exponent_of(g.dc);
+        dct = f32_scaled(g.dc, ex);
+        fx = __shfl_sync(0xffffffffu, Ai.x, lead);
+        if (DIM >= 2) fy = __shfl_sync(0xffffffffu, Ai.y, lead);
+        if (DIM >= 3) fz = __shfl_sync(0xffffffffu, Ai.z, lead);
+      }
+      const float band = 0x1p-12f * dct * dct;
+      auto frame = [&](const V4& R, int relx, int oy, int oz) {
+        float4 S;
+        if constexpr (MIXED) {
+          S.x = R.x + (float)relx * dct;
+          S.y = DIM >= 2 ? R.y + (float)oy * dct : 0.f;
+          S.z = DIM >= 3 ? R.z + (float)oz * dct : 0.f;
+          S.w = R.w;
+        } else {
+          S.x = f32_scaled(R.x - fx, ex);
+          S.y = DIM >= 2 ? f32_scaled(R.y - fy, ex) : 0.f;
+          S.z = DIM >= 3 ? f32_scaled(R.z - fz, ex) : 0.f;
+          S.w = f32_scaled(R.w, ex);
+        }
+        return S;
+      };
+      float4 H = frame(Ai, cx_seg, 0, 0);
+      H.w *= a.kh_f;
+      // the members' bounding box and largest kh d
+      const float inf = __int_as_float(0x7f800000);
+      float bxl = mine ? H.x : inf, bxh = mine ? H.x : -inf, byl = mine ? H.y : inf, byh = mine ? H.y : -inf;
+      float bzl = mine ? H.z : inf, bzh = mine ? H.z : -inf, bkh = mine ? H.w : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        bxl = fminf(bxl, __shfl_xor_sync(0xffffffffu, bxl, o)); bxh = fmaxf(bxh, __shfl_xor_sync(0xffffffffu, bxh, o));
+        if (DIM >= 2) { byl = fminf(byl, __shfl_xor_sync(0xffffffffu, byl, o)); byh = fmaxf(byh, __shfl_xor_sync(0xffffffffu, byh, o)); }
+        if (DIM >= 3) { bzl = fminf(bzl, __shfl_xor_sync(0xffffffffu, bzl, o)); bzh = fmaxf(bzh, __shfl_xor_sync(0xffffffffu, bzh, o)); }
+        bkh = fmaxf(bkh, __shfl_xor_sync(0xffffffffu, bkh, o));
+      }
+      if (!mine) H.x = __int_as_float(0x7fc00000);             // NaN: a lane outside the segment accepts nothing
+      if (mine) {
+        // candidates of the slot's own 3^dim block (sph_pair_counts), and the capacity of its cell
+        const int64_t home = a.grid[b0].cell_off + (int64_t)nx * row0 + cx;
+        if (a.cell_start[home + 1] - a.cell_start[home] > 2048) set_status(a.status, SPH_ERR_CAPACITY);
+      }
+      __syncwarp();
+      for (int r = 0; r < kRows; ++r) {
+        const int64_t rb = __shfl_sync(0xffffffffu, rbase, r);
+        if (rb < 0) continue;                                  // row outside the mesh
+        const int r0 = __shfl_sync(0xffffffffu, rs0, r), r1 = __shfl_sync(0xffffffffu, rs1, r);
+        const int oy = DIM >= 2 ? r % 3 - 1 : 0, oz = DIM >= 3 ? r / 3 - 1 : 0;
+        const int rc = 3 * (oy + 1) + 9 * (oz + 1);            // code of the row's ox = -1 cell
+        if (mine) ncand += (unsigned)(a.cell_start[rb + (cx + 1 < nx ? cx + 2 : nx)] - a.cell_start[rb + (cx > 0 ? cx - 1 : 0)]);
+        for (int base = r0; base < r1; base += 32) {
+          const int j = base + lane;
+          const bool jv = j < r1;
+          const int jl = jv ? j : r0;
+          const int relx = a.slot_cell[jl] - (int)rb - cx0;
+          const float4 S = frame(A[jl], relx, oy, oz);
+          // keep the candidates within reach of the members' box (a superset:
+          // every rounding below is monotone in the distance)
+          const float gx = fmaxf(0.f, fmaxf(S.x - bxh, bxl - S.x));
+          const float gy = DIM >= 2 ? fmaxf(0.f, fmaxf(S.y - byh, byl - S.y)) : 0.f;
+          const float gz = DIM >= 3 ? fmaxf(0.f, fmaxf(S.z - bzh, bzl - S.z)) : 0.f;
+          const float Rm = fmaf(a.kh_f, S.w, bkh);
+          const bool keep = jv && fmaf(-Rm, Rm, Pair<true, DIM>::r2_of(gx, gy, gz)) <= band;
+          const unsigned km = __ballot_sync(0xffffffffu, keep);
+          const int nc = __popc(km);
+          if (keep) {
+            const int c = __popc(km & lt);
+            cand[warp][c] = S;
+            const int off = j - (wide ? __float_as_int(nb_tab[warp][seg][rc + 1 + relx].x) : r0);
+            cand_ent[warp][c] = make_int2(((rc + 1 + relx) << 11) | (off & 2047), j);
+          }
+          // a chunk adds at most nc entries to a list: flush first if one could overflow
+          if (__any_sync(0xffffffffu, cnt > kRowCap - nc)) flush();
+          __syncwarp();
+          const int mybase = cx_seg << 11;
+#pragma unroll 4
+          for (int c = 0; c < nc; ++c) {
+            const float4 Sc = cand[warp][c];
+            const float r2 = Pair<true, DIM>::r2_of(Sc.x - H.x, DIM >= 2 ? Sc.y - H.y : 0.f, DIM >= 3 ? Sc.z - H.z : 0.f);
+            const float R = fmaf(a.kh_f, Sc.w, H.w);
+            const float diff = fmaf(-R, R, r2);              // r^2 - R^2
+            bool acc = diff < 0.f;
+            if (fabsf(diff) <= band) {                        // too close to call in FP32: FP64 decides
+              const int jc = cand_ent[warp][c].y;
+              ++nexact;
+              acc = jc == i || exact_accept(a, DIM, a.perm[i], a.perm[jc]);
+            }
+            if (acc) list[warp][lane][cnt++] = (uint16_t)(cand_ent[warp][c].x - mybase);
+          }
+          __syncwarp();   // the candidate buffer is rewritten by the next chunk
+        }
+      }
+      ++seg;
     }
-    if constexpr (LIST) flush_lists();
-    else if (act) flush();
+    flush();
 
     if constexpr (GRAD) {
       if (act) {
         V4* GP = reinterpret_cast<V4*>(a.gP);
         V4* GV = reinterpret_cast<V4*>(a.gV);
         const T rs = (T)a.rscale;                      // undo the volume and W' scales (powers of two)
-        V4 q{};
-        q.x = gP[0] * rs; q.y = gP[1] * rs; q.z = gP[2] * rs;
-        GP[i] = q;
+        V4 w{};
+        w.x = gP[0] * rs; w.y = gP[1] * rs; w.z = gP[2] * rs;
+        GP[i] = w;
 #pragma unroll
         for (int c = 0; c < DIM; ++c) {
-          V4 g{};
-          g.x = gV[c][0] * rs; g.y = gV[c][1] * rs; g.z = gV[c][2] * rs;
-          GV[(int64_t)c * a.n + i] = g;
+          V4 gr{};
+          gr.x = gV[c][0] * rs; gr.y = gV[c][1] * rs; gr.z = gV[c][2] * rs;
+          GV[(int64_t)c * a.n + i] = gr;
         }
       }
-      __syncwarp();
-      continue;
-    }
-    if constexpr (LIST) {
-      if (act) {
-        if (vc > a.vcap) set_status(a.status, SPH_ERR_CAPACITY);
-        a.vcnt[a.e_of_c ? a.e_of_c[i] : i] = vc < a.vcap ? vc : a.vcap;
-        const int64_t p = a.perm[i];
-        a.vref[p] = a.x[p];
-        if (DIM >= 2) a.vref[a.n + p] = a.y[p];
-        if (DIM >= 3) a.vref[2 * a.n + p] = a.z[p];
-        a.vref[3 * a.n + p] = a.d[p];
-      }
-      __syncwarp();
-      continue;
-    }
-    if constexpr (VJP) {
+    } else if constexpr (VJP) {
       if (act) {
         double* o = a.vjp_out + 11 * (int64_t)a.perm[i];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) { o[q] = (double)s_bx[q].s; o[3 + q] = (double)s_bv[q].s; }
+        for (int k = 0; k < 3; ++k) { o[k] = (double)s_bx[k].s; o[3 + k] = (double)s_bv[k].s; }
         o[6] = (double)s_bP.s;
         o[7] = (double)s_bZ.s;
         o[8] = (double)s_bV.s;
         o[9] = (double)s_bd.s;
         o[10] = (double)s_brho.s;
       }
-      __syncwarp();
-      continue;
+    } else {
+      if (act) {
+        nfull -= 1;   // the self pair
+        fw.fold();
+        fw.write(a, i, nfull);
+      }
+      warp_counters(a, act, nfull, ncand, MIXED ? nexact : 0u, ui, lane,
+                    a.load_timed ? (unsigned)(clock64() - t_start) : 0u);
     }
-    if (act) {
-      nfull -= 1;   // the self pair
-      fw.fold();
-      fw.write(a, i, nfull);
-    }
-    warp_counters(a, act, nfull, ncand, nexact, ui, lane,
-                  a.load_timed ? (unsigned)(clock64() - t_start) : 0u);
-    __syncwarp();   // the home buffer is rewritten by the next chunk of home particles
-  }
-  __syncwarp();     // the neighbour-start buffer is rewritten by the next cell
+    __syncwarp();     // the segment tables and lists are rewritten by the next group
+    if (lane == 0) q = atomicAdd(a.work_counter, 1ull) + (unsigned long long)gridDim.x * kWarps;
+    q = __shfl_sync(0xffffffffu, q, 0);
   }
 }
 
 // Persistent grid: SMs x resident CTAs per SM, capped by the handle's
-// pair_blocks_per_sm (0 = as many as fit).
+// pair_blocks_per_sm (0 = as many as fit) and by the number of groups.
+// Groups hold 32 slots; a system too small to give every SM four warps takes
+// 16 or 8 slots per group, so that more SMs share its scan.
 template <bool MIXED, int DIM, int MODE, bool HLL, bool EXTRA = true>
 cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
   static int sms = 0, per_sm = 0;
@@ -550,8 +493,13 @@ cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<MIXED, DIM, MODE, HLL, EXTRA>, kPairBlock, 0);
     if (per_sm < 1) per_sm = 1;
   }
+  PairArgs a = args;
+  a.group = 32;
+  while (a.group > 8 && a.n < (int64_t)4 * sms * a.group) a.group >>= 1;
+  const int64_t groups = (a.n + a.group - 1) / a.group;
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
-  return launch_chained(k_pair<MIXED, DIM, MODE, HLL, EXTRA>, dim3(sms * b), dim3(kPairBlock), st, args);
+  const int grid = groups < (int64_t)sms * b ? (int)groups : sms * b;
+  return launch_chained(k_pair<MIXED, DIM, MODE, HLL, EXTRA>, dim3(grid), dim3(kPairBlock), st, a);
 }
 
 template <bool MIXED, int MODE, bool HLL, bool EXTRA>
@@ -604,29 +552,6 @@ cudaError_t launch_pair_vjp(sph_handle* h, const sph_state& s, const void* G, co
   cudaError_t e = cudaMemsetAsync(&h->counters[5], 0, sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   e = fp64 ? launch_dim<false, kModeVjp>(h, a, st) : launch_dim<true, kModeVjp>(h, a, st);
-  h->launches += 1;
-  return e;
-}
-
-// Verlet list build: the pair kernel over the radius (1 + beta) kappa h_ij;
-// returns at once on the device unless vflag[0] is set.
-cudaError_t launch_list_build(sph_handle* h, const sph_state& s, cudaStream_t st) {
-  PairArgs a = make_args(h, s);
-  a.K = 0;
-  a.collect_adj = 0;
-  a.pair_i = a.pair_j = nullptr;
-  const double khl = h->dp.kh * (1.0 + h->dp.cell_beta);
-  a.kh = khl;
-  a.kh_f = (float)khl;
-  if (h->unit_sched != SPH_SCHED_GLOBAL) {   // rows and entries in the unit-major evaluation order
-    a.e_of_c = h->e_of_c;
-    a.Ac = h->packAc;
-  }
-  // work counter zeroed by the step's k_pack (launch_pack with list_counters)
-  a.work_counter = &h->counters[7];
-  a.vinst = h->n_inst > 1 ? h->vinst : nullptr;   // only the instances whose lists are rebuilt
-  cudaError_t e = h->dp.precision == SPH_PREC_MIXED ? launch_dim<true, kModeList>(h, a, st)
-                                                    : launch_dim<false, kModeList>(h, a, st);
   h->launches += 1;
   return e;
 }

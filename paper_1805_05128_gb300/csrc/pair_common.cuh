@@ -15,7 +15,6 @@ namespace {
 struct PairArgs {
   int64_t n;
   const int64_t* total_cells_dev;
-  int64_t total_cells;   // read from total_cells_dev by the kernel
   int n_inst;
   const int64_t* inst_off;
   const GridInfo* grid;
@@ -41,6 +40,7 @@ struct PairArgs {
   unsigned long long* counters;
   int* status;
   unsigned long long* work_counter;   // next cell for the persistent warps (zeroed per launch)
+  int group;                           // k_pair: slots per warp and group (at most 32)
   const int* vinst;                    // list build: the instances rebuilt in this step, or NULL (all)
   int collect_adj;   // record unit adjacency in this evaluation
   int load_timed;    // unit loads in SM cycles (SPH_LOAD_TIME) instead of pair counts
@@ -57,7 +57,7 @@ struct PairArgs {
   const void* G;
   const void* GR2;
   double* vjp_out;
-  // Verlet lists (k_pair in list mode writes them, k_pair_lists reads them)
+  // Verlet lists (k_list_build writes them, k_pair_lists reads them)
   uint32_t* vlist;   // [n][vcap]: (slot j << 5) | neighbour-cell code, particle-major
   int32_t* vcnt;
   double* vref;      // x, y, z, d per particle at the build (4 arrays of n)
@@ -102,9 +102,8 @@ struct PairArgs {
 
 constexpr int kModeFwd = 0;    // rates
 constexpr int kModeVjp = 1;    // reverse mode of the rates
-constexpr int kModeList = 2;   // Verlet list build over the (1 + beta) radius
-constexpr int kModeGrad = 3;   // SPH gradients of P and v (order-2 reconstruction)
-constexpr int kModeFwd2 = 4;   // rates with states reconstructed to the pair midpoint
+constexpr int kModeGrad = 2;   // SPH gradients of P and v (order-2 reconstruction)
+constexpr int kModeFwd2 = 3;   // rates with states reconstructed to the pair midpoint
 
 template <bool MIXED>
 struct Ops;
@@ -747,7 +746,6 @@ PairArgs make_args(sph_handle* h, const sph_state& s) {
   PairArgs a{};
   a.n = h->n;
   a.total_cells_dev = h->total_cells;
-  a.total_cells = 0;
   a.n_inst = h->n_inst;
   a.inst_off = h->inst_off;
   a.grid = h->grid;

@@ -91,6 +91,46 @@ __host__ __device__ __forceinline__ double f64_of(float f) {
 #endif
 }
 
+// Unbiased exponent of a positive normal double.
+__host__ __device__ __forceinline__ int exponent_of(double x) {
+#ifdef __CUDA_ARCH__
+  return ((__double2hiint(x) >> 20) & 0x7ff) - 1023;
+#else
+  unsigned long long bb;
+  memcpy(&bb, &x, 8);
+  return (int)((bb >> 52) & 0x7ff) - 1023;
+#endif
+}
+
+// x 2^-e rounded to FP32 (to nearest, ties away), on the integer ALU: the FP32
+// frame of the pair search of FP64 handles, e the exponent of the cell edge, so
+// that lengths of any unit stay in FP32's range.  Below 2^-125 the result is 0,
+// from 2^127 up it is infinite; NaN stays NaN.
+__host__ __device__ __forceinline__ float f32_scaled(double x, int e) {
+#ifdef __CUDA_ARCH__
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+#else
+  unsigned long long bb;
+  memcpy(&bb, &x, 8);
+  const unsigned hi = (unsigned)(bb >> 32), lo = (unsigned)bb;
+#endif
+  const unsigned h = hi & 0x7fffffffu;
+  const int E = (int)(h >> 20) - e;
+  unsigned r;
+  if (h >= 0x7ff00000u) r = (h > 0x7ff00000u || lo) ? 0x7fc00000u : 0x7f800000u;
+  else if (E < 898 || (h >> 20) == 0u) r = 0u;
+  else if (E > 1149) r = 0x7f800000u;
+  else r = ((h - ((unsigned)(896 + e) << 20)) << 3) + (lo >> 29) + ((lo >> 28) & 1u);
+  r |= hi & 0x80000000u;
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(r);
+#else
+  float f;
+  memcpy(&f, &r, 4);
+  return f;
+#endif
+}
+
 // Reference velocity of a mixed pack: t = trunc(v) with |t| <= 32767, built
 // from v's bits by integer operations (no FP64 arithmetic), and k = t as an
 // int.  v - t is then exact in FP64 (|v - t| < 1 unless clamped) and rounds
