@@ -298,35 +298,6 @@ __device__ __forceinline__ void eos(const Mat& m, double rho, double e, double& 
   c = c2 > 0.0 ? sqrt(c2) : 0.0;
 }
 
-// dW/dr of the cubic spline (support 2h) or the Wendland C2 kernel (support
-// kappa h), for dimension DIM.
-template <typename T, int DIM>
-__device__ __forceinline__ T kernel_dw(int kernel, T kappa, T r, T h) {
-  const T pi = T(3.14159265358979323846);
-  if (kernel == SPH_KERNEL_CUBIC) {
-    T ih = T(1) / h;
-    T q = r * ih;
-    T norm;
-    if (DIM == 1) norm = T(2.0 / 3.0) * ih * ih;
-    else if (DIM == 2) norm = T(10) / (T(7) * pi) * ih * ih * ih;
-    else norm = ih * ih * ih * ih / pi;
-    T f;
-    if (q < T(1)) f = q * (T(2.25) * q - T(3));
-    else if (q < T(2)) { T t = T(2) - q; f = T(-0.75) * t * t; }
-    else f = T(0);
-    return norm * f;
-  } else {
-    T H = kappa * h;
-    T iH = T(1) / H;
-    T s = r * iH;
-    if (s >= T(1)) return T(0);
-    T t = T(1) - s;
-    if (DIM == 1) return T(1.25) * iH * iH * (T(-12) * s * t * t);
-    T norm = (DIM == 2) ? T(7) / pi * iH * iH * iH : T(21) / (T(2) * pi) * iH * iH * iH * iH;
-    return norm * (T(-20) * s * t * t * t);
-  }
-}
-
 // --------------------------------------------------------------------------
 // Programmatic dependent launch of a step's kernels: each is launched while
 // its predecessor in the stream still runs (launch_chained), so that the

@@ -142,14 +142,14 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         dy = DIM >= 2 ? __dsub_rn(Aj.y, Ai.y) : 0.0;
         dz = DIM >= 3 ? __dsub_rn(Aj.z, Ai.z) : 0.0;
       }
-      const T r2 = P::r2_of(dx, dy, dz);
-      if (!(r2 > T(0))) return;
-      const T ir = rsqrt_(r2);
-      const T r = r2 * ir;
+      const T r2 = MIXED ? P::r2_of(dx, dy, dz) : fw.r2_fused(dx, dy, dz);
+      if (!positive(r2)) return;
+      T ir, r;
+      rsqrt_sqrt(r2, ir, r);
       const T e[3] = {dx * ir, dy * ir, dz * ir};
-      const T hij = (MIXED ? (T)a.eta_half_f : (T)a.eta_half) * (Ai.w + Aj.w);
-      const T w = -(MIXED ? dw_fast<T, DIM>(a.kernel, (T)a.kappa_f, r, hij, (T)a.wscale_f)
-                          : kernel_dw<T, DIM>(a.kernel, (T)a.kappa, r, hij));
+      T w;
+      if constexpr (MIXED) w = -dw_fast<T, DIM>(a.kernel, (T)a.kappa_f, r, (T)a.eta_half_f * (Ai.w + Aj.w), (T)a.wscale_f);
+      else w = -dw64<DIM, -1>(a.kernel, a.kappa, a.eta_half, r, Ai.w + Aj.w);
       const T f = Bj.w * w;
       const T dP = Cj.x - Ci.x;
       T dv[3];
@@ -192,10 +192,10 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         dy = DIM >= 2 ? __dsub_rn(Aj.y, Ai.y) : 0.0;
         dz = DIM >= 3 ? __dsub_rn(Aj.z, Ai.z) : 0.0;
       }
-      const T r2 = P::r2_of(dx, dy, dz);
-      if (!(r2 > T(0))) return;
-      const T ir = rsqrt_(r2);
-      const T r = r2 * ir;
+      const T r2 = MIXED ? P::r2_of(dx, dy, dz) : fw.r2_fused(dx, dy, dz);
+      if (!positive(r2)) return;
+      T ir, r;
+      rsqrt_sqrt(r2, ir, r);
       const T e[3] = {dx * ir, dy * ir, dz * ir};
       T vi[3] = {Bi.x, Bi.y, Bi.z}, vj[3] = {Bj.x, Bj.y, Bj.z};
       if constexpr (MIXED) {   // lab-frame velocities: relative ones plus the references
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       for (int q = 0; q < DIM; ++q) { vRi += vi[q] * e[q]; vRj += vj[q] * e[q]; }
       const T Zi = Ci.y, Zj = Cj.y, zs = Zi + Zj, Pi = Ci.x, Pj = Cj.x;
       T Ps, vs, izs = T(0);
-      if (zs > T(0)) {
+      if (positive(zs)) {
         izs = rcp_(zs);
         Ps = (Zj * Pi + Zi * Pj + Zi * Zj * (vRi - vRj)) * izs;
         vs = (Zi * vRi + Zj * vRj + Pi - Pj) * izs;
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       s_bV.add(gF * T(2) * Vj * Ps * W - GRj * T(2) * rhoj * (vs - vRj) * W);
       s_brho.add(-(GRi * T(2) * Vj * (vRi - vs) * W));
       T gPi, gZi = T(0);
-      if (zs > T(0)) {
+      if (positive(zs)) {
         gPi = (gPs * Zj + gvs) * izs;
         gvRi += (gPs * Zi * Zj + gvs * Zi) * izs;
         gvRj += (gvs * Zj - gPs * Zi * Zj) * izs;
