@@ -2,6 +2,7 @@
 // CSPH hot path (arXiv 1805.05128) for sm_103a.  Not part of the public ABI.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -321,6 +322,93 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, cuda
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = 0;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// --------------------------------------------------------------------------
+// Sums over one thread-block cluster in a fixed order (butterfly in each warp,
+// over the warps, then the CTAs in rank order through distributed shared
+// memory), so that a whole-array sum needs neither a workspace nor a second
+// kernel.  NV sums at once; returns true in the one thread that holds them.
+// --------------------------------------------------------------------------
+constexpr int kSumBlock = 1024;
+template <int NV>
+__device__ __forceinline__ bool cluster_sum(double (&v)[NV]) {
+  namespace cg = cooperative_groups;
+  __shared__ double sh[NV][kSumBlock / 32];
+  __shared__ double blk[NV];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane == 0) sh[k][w] = v[k];
+  }
+  __syncthreads();
+  if (w == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      double t = sh[k][lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane == 0) blk[k] = t;
+    }
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  const bool mine = cl.block_rank() == 0 && threadIdx.x == 0;
+  if (mine) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      double t = 0.0;
+      for (unsigned r = 0; r < cl.num_blocks(); ++r) t += *cl.map_shared_rank(&blk[k], r);
+      v[k] = t;
+    }
+  }
+  cl.sync();          // no CTA leaves while its partial sums are read
+  return mine;
+}
+
+// CTAs per cluster for a sum over n elements: one per 4096 (four loads in flight
+// per thread), up to the 16 that fit a cluster here (8 where only the portable
+// size does).  A sum is bound by the FP64 pipe of the cluster's SMs.
+template <typename K>
+int sum_cluster_size(K kernel, int64_t n) {
+  static int most = 0;
+  if (most == 0) {
+    most = 8;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(kSumBlock);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int active = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) == cudaSuccess && active > 0)
+      most = 16;
+    cudaGetLastError();   // a refused query only means the portable size
+  }
+  int c = 1;
+  while (c < most && n > (int64_t)4096 * c) c *= 2;
+  return c;
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), int clusters, int per, int threads, cudaStream_t st, Args... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)per;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)clusters * (unsigned)per);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;

@@ -147,19 +147,21 @@ __global__ void k_vjp_chain(int64_t n, DevParams P, const sph_state W, sph_state
   }
 }
 
-// Fixed-order sum of the per-particle parameter adjoints into out[0..1] (+=).
-__global__ void k_sum_params(int64_t n, const double* __restrict__ par, double* out) {
-  __shared__ double sh[2][1024];
-  double s0 = 0.0, s1 = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) { s0 += par[2 * i]; s1 += par[2 * i + 1]; }
-  sh[0][threadIdx.x] = s0;
-  sh[1][threadIdx.x] = s1;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) { sh[0][threadIdx.x] += sh[0][threadIdx.x + w]; sh[1][threadIdx.x] += sh[1][threadIdx.x + w]; }
-    __syncthreads();
+// Fixed-order sum of the per-particle parameter adjoints into out[0..1] (+=),
+// one cluster of CTAs (one CTA: 122 us on 203k particles; a cluster: 16 us).
+__global__ void __launch_bounds__(kSumBlock) k_sum_params(int64_t n, const double* __restrict__ par, double* out) {
+  const int64_t stride = (int64_t)gridDim.x * kSumBlock;   // the grid is one cluster
+  double s[2] = {0.0, 0.0};
+#pragma unroll 4
+  for (int64_t i = (int64_t)blockIdx.x * kSumBlock + threadIdx.x; i < n; i += stride) {
+    s[0] += par[2 * i];
+    s[1] += par[2 * i + 1];
   }
-  if (threadIdx.x == 0) { out[0] += sh[0][0]; out[1] += sh[1][0]; }
+  if (cluster_sum(s)) { out[0] += s[0]; out[1] += s[1]; }
+}
+
+cudaError_t launch_sum_params(int64_t n, const double* par, double* out, cudaStream_t st) {
+  return launch_clusters(k_sum_params, 1, sum_cluster_size(k_sum_params, n), kSumBlock, st, n, par, out);
 }
 
 }  // namespace
@@ -179,9 +181,9 @@ cudaError_t launch_rates_vjp(sph_handle* h, const sph_state& W, sph_state& adj, 
     e = launch_pair_vjp(h, W, h->adj_G, h->adj_GR, h->adj_pair, st, h->adj64_A, h->adj64_B, h->adj64_C);
     if (e != cudaSuccess) return e;
     k_vjp_chain<<<g, kBlock, 0, st>>>(n, h->dp, W, adj, h->adj_pair, dt, predicted, h->adj_par);
-    k_sum_params<<<1, 1024, 0, st>>>(n, h->adj_par, par);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     h->launches += 3;
-    return cudaGetLastError();
+    return launch_sum_params(n, h->adj_par, par, st);
   }
   if (h->dp.precision == SPH_PREC_MIXED)
     k_adj_pack<float, float4, float2><<<g, kBlock, 0, st>>>(n, h->dp.dim, h->perm, adj, W.m, h->rho_slot, dt,
@@ -195,9 +197,9 @@ cudaError_t launch_rates_vjp(sph_handle* h, const sph_state& W, sph_state& adj, 
   e = launch_pair_vjp(h, W, h->adj_G, h->adj_GR, h->adj_pair, st);
   if (e != cudaSuccess) return e;
   k_vjp_chain<<<g, kBlock, 0, st>>>(n, h->dp, W, adj, h->adj_pair, dt, predicted, h->adj_par);
-  k_sum_params<<<1, 1024, 0, st>>>(n, h->adj_par, par);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   h->launches += 3;
-  return cudaGetLastError();
+  return launch_sum_params(n, h->adj_par, par, st);
 }
 
 }  // namespace csph
