@@ -172,10 +172,12 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
             if (__any_sync(0xffffffffu, cnt > kBuildCap - 32)) flush_lists();
             const int j = base + lane;
             const bool jv = j < r1;
-            const int ox = j < s_0 ? -1 : (j < b1 ? 0 : 1);
-            const float4 S = frame(A[jv ? j : r0], ox, oy, oz);
+            const V4 R = A[jv ? j : r0];
+            float4 S{};
             uint32_t ent = 0;
             if (jv) {
+              const int ox = j < s_0 ? -1 : (j < b1 ? 0 : 1);
+              S = frame(R, ox, oy, oz);
               const int off = j - (ox < 0 ? s_m : (ox == 0 ? s_0 : b1));
               if (off > 2047) set_status(a.status, SPH_ERR_CAPACITY);   // cell over 2047 particles
               ent = ((uint32_t)(rc + ox + 1) << 11) | (uint32_t)(off & 2047);

@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
   const int half = lane / kSlotLanes, hl = lane % kSlotLanes;   // the slot's group of lanes, lane in it
   const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
   // Work partition.  SPH_SCHED_GLOBAL: groups of 32 consecutive slots from one
-  // global counter.  Units: each unit owns a contiguous range of evaluation
+  // global counter, the last ones of 8 (launch_lists_one).  Units: each unit owns a contiguous range of evaluation
   // slots and a counter; CTA b starts on unit b K / gridDim.x (the CTAs are
   // spread evenly over the units), takes groups of 32 slots of that unit and,
   // with SPH_SCHED_UNITS, moves on to the following units once it is drained
@@ -122,11 +122,14 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
     int g0 = 0, g1 = 0;
     if (a.unit_sched == SPH_SCHED_GLOBAL) {
       unsigned long long gw = 0;
-      if (lane == 0) gw = atomicAdd(a.work_counter, 32ull);
+      if (lane == 0) gw = atomicAdd(a.work_counter, 1ull);
       gw = __shfl_sync(0xffffffffu, gw, 0);
-      if ((int64_t)gw >= a.n) break;
-      g0 = (int)gw;
-      g1 = (int64_t)g0 + 32 < a.n ? g0 + 32 : (int)a.n;
+      const bool big = (int64_t)gw < a.big_groups;
+      const int64_t at = big ? a.big * (int64_t)gw : a.big * a.big_groups + kSlotsPerWarp * ((int64_t)gw - a.big_groups);
+      if (at >= a.n) break;
+      g0 = (int)at;
+      const int64_t end = at + (big ? a.big : kSlotsPerWarp);
+      g1 = end < a.n ? (int)end : (int)a.n;
     } else {
       int ok = 0;
       if (lane == 0) {
@@ -351,8 +354,16 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       }
     }
     if constexpr (STAGE) cp_wait<0>();              // the last slot's stand-in copy, before the stages are reused
-    if (a.K > 0 && hl == 0 && unit_run >= 0 && unit_load)
-      atomicAdd(&a.load_acc[unit_run], (unsigned long long)unit_load);
+    if (a.K > 0) {
+      // one atomic for the group where all its slots belong to one unit (the usual case)
+      const int u0 = __shfl_sync(0xffffffffu, unit_run, 0);
+      if (__all_sync(0xffffffffu, unit_run < 0 || unit_run == u0)) {
+        const unsigned sum = __reduce_add_sync(0xffffffffu, hl == 0 ? unit_load : 0u);
+        if (lane == 0 && u0 >= 0 && sum) atomicAdd(&a.load_acc[u0], (unsigned long long)sum);
+      } else if (hl == 0 && unit_run >= 0 && unit_load) {
+        atomicAdd(&a.load_acc[unit_run], (unsigned long long)unit_load);
+      }
+    }
     __syncwarp();
     {
       const int64_t i = g0 + lane;                     // one slot of the group per lane
@@ -451,7 +462,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
 }
 
 template <bool MIXED, int DIM, bool HLL, bool EXTRA, bool STAGE, int KERN>
-cudaError_t launch_lists_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
+cudaError_t launch_lists_one(const PairArgs& args_in, int blocks_per_sm, cudaStream_t st) {
   static int sms = 0, per_sm = 0;
   if (sms == 0) {
     int dev = 0;
@@ -463,6 +474,20 @@ cudaError_t launch_lists_one(const PairArgs& args, int blocks_per_sm, cudaStream
   }
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
   int grid = sms * b;
+  // Groups of 32 slots share the set-up and the FP64 rate formation best (a
+  // group of 8 costs ~20 % more per slot on a full chip), but a launch ends when
+  // its last groups do.  Up to 27 slots per resident warp every group would be
+  // the last one of its warp: groups of 8 (one pass of the warp, four lanes per
+  // slot), above 16 slots per warp those go out last, after groups of 16.
+  // Beyond, the last 16 slots per warp go out in groups of 8 unless a last wave
+  // of 32 would be full anyway (by 5/6).  List kernel against 32 throughout,
+  // 4256 warps, no units: 9k 82 -> 33 us, 32k 88 -> 44, 77k 98 -> 71, 140k 125 ->
+  // 107, 203k 159 -> 143, 387k 256 -> 246, 874k 539 -> 530, 1.125M 677 -> 671.
+  PairArgs args = args_in;
+  const int64_t warps = (int64_t)kWarps * grid, n = args.n;
+  args.big = n > 27 * warps ? 32 : 16;
+  const bool full_wave = args.big == 32 && (n + 31) % (32 * warps) >= 32 * warps * 5 / 6;
+  args.big_groups = full_wave ? n / 32 + 1 : (n > 16 * warps ? (n - 16 * warps) / args.big : 0);
   if (args.unit_sched == SPH_SCHED_UNITS_OWNED && args.K > 0)   // the same number of CTAs for every unit
     grid = args.K * (grid / args.K > 0 ? grid / args.K : 1);
   // A plain launch, not chained to the list build before it: chained, the

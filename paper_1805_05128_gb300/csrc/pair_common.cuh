@@ -41,6 +41,8 @@ struct PairArgs {
   int* status;
   unsigned long long* work_counter;   // next cell for the persistent warps (zeroed per launch)
   int group;                           // k_pair: slots per warp and group (at most 32)
+  int big;                             // k_pair_lists: slots of a big group (at most 32)
+  int64_t big_groups;                  // big groups; the slots after them go out in groups of 8
   const int* vinst;                    // list build: the instances rebuilt in this step, or NULL (all)
   int collect_adj;   // record unit adjacency in this evaluation
   int load_timed;    // unit loads in SM cycles (SPH_LOAD_TIME) instead of pair counts
