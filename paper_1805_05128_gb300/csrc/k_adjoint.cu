@@ -29,7 +29,7 @@ namespace csph {
 namespace {
 
 // Adjoint operands in slot order, in the pair kernel's precision T:
-// G = (dL/da' / m, dL/ddE' / m), GR2 = (dL/ddrho', rho of the slot).
+// G = (dL/da' / m, dL/ddE' / m), GR2 = (dL/ddrho', rho of the slot; in FP64 rho dL/ddrho').
 // With predicted = 1 the rates are those after a step: their adjoints are the
 // incoming ones plus h times the adjoints of v', E', rho' (v' = v^h + h a').
 template <typename T, typename V4, typename V2>
@@ -51,7 +51,8 @@ __global__ void k_adj_pack(int64_t n, int dim, const int32_t* __restrict__ perm,
   G[sl] = g;
   V2 r;
   r.x = (T)(adj.drho[p] + hdt * adj.rho[p]);
-  r.y = (T)rho_slot[sl];
+  const double rho = rho_slot[sl];
+  r.y = sizeof(T) == 8 ? (T)(rho * (double)r.x) : (T)rho;
   GR2[sl] = r;
 }
 

@@ -341,8 +341,17 @@ __device__ __forceinline__ void cubic_dw3(T r, T h, T& w, T& wr, T& wh) {
   else if (DIM == 2) norm = T(10.0 / (7.0 * 3.14159265358979323846)) * ih * ih * ih;
   else norm = T(1.0 / 3.14159265358979323846) * (ih * ih) * (ih * ih);
   const T t = T(2) - q;
-  const T g = q < T(1) ? q * (T(2.25) * q - T(3)) : (q < T(2) ? T(-0.75) * t * t : T(0));
-  const T gp = q < T(1) ? T(4.5) * q - T(3) : (q < T(2) ? T(1.5) * t : T(0));
+  const T g_in = q * (T(2.25) * q - T(3)), g_out = T(-0.75) * t * t;
+  const T gp_in = T(4.5) * q - T(3), gp_out = T(1.5) * t;
+  T g, gp;
+  if constexpr (sizeof(T) == 8) {   // the branch on the bits of q >= 0, not on the FP64 pipe
+    const int hq = __double2hiint(q);
+    g = hq < 0x3ff00000 ? g_in : (hq < 0x40000000 ? g_out : T(0));
+    gp = hq < 0x3ff00000 ? gp_in : (hq < 0x40000000 ? gp_out : T(0));
+  } else {
+    g = q < T(1) ? g_in : (q < T(2) ? g_out : T(0));
+    gp = q < T(1) ? gp_in : (q < T(2) ? gp_out : T(0));
+  }
   w = norm * g;
   const T nh = norm * ih;
   wr = nh * gp;
