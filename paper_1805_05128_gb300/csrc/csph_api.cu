@@ -79,7 +79,7 @@ int check_adjoint_state(sph_handle* h, const sph_state* a) {
 }
 
 int eval_rates_impl(sph_handle* h, sph_state* s, cudaStream_t st) {
-  CK(h, launch_derive_dt(h, *s, true, st));
+  CK(h, launch_derive(h, *s, st));
   CK(h, launch_build_grid(h, *s, st));
   CK(h, launch_pack(h, *s, false, st));
   CK(h, launch_pair(h, *s, st));
@@ -413,7 +413,7 @@ int sph_build_cells(sph_handle* h, sph_state* s, void* stream) {
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   h->last_stream = st;
-  CK(h, launch_derive_dt(h, *s, true, st));
+  CK(h, launch_derive(h, *s, st));
   CK(h, launch_build_grid(h, *s, st));
   CK(h, launch_renumber(h, *s, st));
   return SPH_OK;
@@ -439,14 +439,12 @@ int sph_step(sph_handle* h, sph_state* s, int n_steps, double* t_dev, void* stre
   }
   const bool vd3 = h->K > 0 && h->p.n_upd > 0;
   sph_balance_params bp{h->p.theta, h->p.sigma, h->p.gamma_b, h->p.beta_sh};
-  bool dt_from_key = false;   // the previous step's fused second kick left the CFL keys
   for (int k = 0; k < n_steps; ++k) {
     // the CFL minima of the step's start state: from the previous step's second
     // kick inside this call (renumbering permutes an instance's particles and
-    // leaves its minimum unchanged), else a k_derive pass
-    if (k == 0) CK(h, launch_derive_dt(h, *s, false, st));
-    CK(h, launch_reduce_dt(h, st, dt_from_key));
-    CK(h, launch_kick_drift(h, *s, st));
+    // leaves its minimum unchanged), else a pass of its own
+    if (k == 0) CK(h, launch_cfl(h, *s, st));
+    CK(h, launch_kick_drift(h, *s, st, true));
     if (h->verlet) {
       // Verlet lists: the mesh, slot order and lists are rebuilt only when the device flag
       // says so (validity criterion failed or lists invalidated); the kernels read the flag
@@ -457,7 +455,7 @@ int sph_step(sph_handle* h, sph_state* s, int n_steps, double* t_dev, void* stre
     } else {
       CK(h, launch_build_grid(h, *s, st));
     }
-    CK(h, launch_pack(h, *s, true, st, h->verlet && h->unit_sched != SPH_SCHED_GLOBAL, h->verlet));
+    CK(h, launch_pack(h, *s, true, st, h->verlet && h->unit_sched != SPH_SCHED_GLOBAL));
     // unit adjacency is needed only from the evaluation that precedes a rebalance
     h->collect_adj = !vd3 || h->steps_since_balance + 1 >= h->p.n_upd;
     const bool next_dt = k + 1 < n_steps;
@@ -466,11 +464,9 @@ int sph_step(sph_handle* h, sph_state* s, int n_steps, double* t_dev, void* stre
       // list kernel's rate write
       CK(h, launch_list_build(h, *s, st));
       CK(h, launch_pair_lists(h, *s, st, true, t_dev, next_dt));
-      dt_from_key = next_dt;
     } else {
       CK(h, launch_pair(h, *s, st));
       CK(h, launch_kick2(h, *s, t_dev, st, next_dt));
-      dt_from_key = false;
     }
     h->collect_adj = true;
     if (vd3 && ++h->steps_since_balance >= h->p.n_upd) {
@@ -583,8 +579,8 @@ int sph_cfl_dt(sph_handle* h, const sph_state* s, double* dt_out, void* stream) 
   if (!dt_out) return fail(h, SPH_ERR_INVALID, "dt_out is NULL");
   cudaStream_t st = (cudaStream_t)stream;
   h->last_stream = st;
-  CK(h, launch_derive_dt(h, *s, false, st));
-  CK(h, launch_reduce_dt(h, st, false));
+  CK(h, launch_cfl(h, *s, st));
+  CK(h, launch_reduce_dt(h, st));
   CK(h, cudaMemcpyAsync(dt_out, h->dt, sizeof(double) * h->n_inst, cudaMemcpyDeviceToDevice, st));
   return SPH_OK;
 }
@@ -679,7 +675,7 @@ int sph_cell_index(sph_handle* h, const sph_state* s, int32_t* cell_out, double*
   cudaStream_t st = (cudaStream_t)stream;
   h->last_stream = st;
   sph_state tmp = *s;
-  CK(h, launch_derive_dt(h, tmp, true, st));
+  CK(h, launch_derive(h, tmp, st));
   CK(h, launch_build_grid(h, tmp, st));
   std::vector<GridInfo> g(h->n_inst);
   CK(h, cudaMemcpyAsync(g.data(), h->grid, sizeof(GridInfo) * h->n_inst, cudaMemcpyDeviceToHost, st));
@@ -844,20 +840,20 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
       CK(h, launch_pack_fp64(h, W, true, h->adj64_A, h->adj64_B, h->adj64_C, h->adj64_rho, st));
       CK(h, launch_rates_vjp(h, W, *adj_in, ck->dt + k, 1, adj_params, st, true));
     } else {
-      CK(h, launch_pack(h, W, true, st));
+      CK(h, launch_pack(h, W, true, st, false, true));
       CK(h, launch_rates_vjp(h, W, *adj_in, ck->dt + k, 1, adj_params, st));
     }
   }
   if (ck->rates_from_state) {
     // the held rates at the checkpoint were evaluated at its own state
     CK(h, copy_dynamic(W, ck->state, n, st));
-    CK(h, launch_derive_dt(h, W, true, st));
+    CK(h, launch_derive(h, W, st));
     CK(h, launch_build_grid(h, W, st));
     if (rev64) {
       CK(h, launch_pack_fp64(h, W, false, h->adj64_A, h->adj64_B, h->adj64_C, h->adj64_rho, st));
       CK(h, launch_rates_vjp(h, W, *adj_in, h->dt, 0, adj_params, st, true));
     } else {
-      CK(h, launch_pack(h, W, false, st));
+      CK(h, launch_pack(h, W, false, st, false, true));
       CK(h, launch_rates_vjp(h, W, *adj_in, h->dt, 0, adj_params, st));
     }
   }

@@ -38,7 +38,6 @@ struct GridInfo {
 struct BlockPart {
   long long lo[3], hi[3];  // bounding box
   long long d1, d2;        // two largest particle sizes
-  long long dtmin;         // min_i eta d_i / (c_i + |v_i|)
 };
 
 // Verlet lists: the grid-wide maximum of the validity criterion and the box
@@ -160,7 +159,8 @@ struct sph_handle {
   void* packC = nullptr;
   double* rho_slot = nullptr;        // [n] density of slot s (FP64)
 
-  long long* dt_key = nullptr;             // [n_inst] CFL keys left by the fused second kick
+  long long* dt_key = nullptr;             // [n_inst] CFL keys: LLONG_MAX between an accumulation (k_cfl, the
+                                           // second kick) that the kick-drift has read and the next one
   double* dmax_nbr = nullptr;        // [n] largest neighbour size of particle p (last evaluation)
 
   // Voronoi work units
@@ -372,31 +372,32 @@ __device__ __forceinline__ bool cluster_sum(double (&v)[NV]) {
   return mine;
 }
 
-// CTAs per cluster for a sum over n elements: one per 4096 (four loads in flight
-// per thread), up to the 16 that fit a cluster here (8 where only the portable
-// size does).  A sum is bound by the FP64 pipe of the cluster's SMs.
+// CTAs in a cluster for work on n elements, one per `each` of them: up to the 16
+// that fit a cluster here (8 where only the portable size does).  (A sum is
+// bound by the FP64 pipe of the cluster's SMs.)
 template <typename K>
-int sum_cluster_size(K kernel, int64_t n) {
+int cluster_size_for(K kernel, int threads, int64_t n, int64_t each) {
   static int most = 0;
   if (most == 0) {
-    most = 8;
+    int m = 8;
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 16;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3(kSumBlock);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int active = 0;
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
         cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) == cudaSuccess && active > 0)
-      most = 16;
+      m = 16;
     cudaGetLastError();   // a refused query only means the portable size
+    most = m;
   }
   int c = 1;
-  while (c < most && n > (int64_t)4096 * c) c *= 2;
+  while (c < most && n > each * c) c *= 2;
   return c;
 }
 
@@ -425,22 +426,25 @@ void set_global_error(const std::string& msg);
 
 // Launchers (defined in k_step.cu, k_pair.cu, k_vd3.cu).  They enqueue on
 // `st` and return the launch status.
-cudaError_t launch_derive_dt(sph_handle* h, const sph_state& s, bool with_bbox, cudaStream_t st);
-// from_key: the step's dt from the CFL keys that the previous step's fused second
-// kick left in dt_key (else from the block partials); dt_key is reset either way
-cudaError_t launch_reduce_dt(sph_handle* h, cudaStream_t st, bool from_key = false);
-cudaError_t launch_kick_drift(sph_handle* h, const sph_state& s, cudaStream_t st);
+// d, P, c and the block partials (bounding box, sizes) of a mesh build at the current state
+cudaError_t launch_derive(sph_handle* h, const sph_state& s, cudaStream_t st);
+// the CFL keys of the current state into dt_key
+cudaError_t launch_cfl(sph_handle* h, const sph_state& s, cudaStream_t st);
+// dt from the CFL keys, which are reset
+cudaError_t launch_reduce_dt(sph_handle* h, cudaStream_t st);
+// from_key: the step's dt from the CFL keys (else h->dt as it is)
+cudaError_t launch_kick_drift(sph_handle* h, const sph_state& s, cudaStream_t st, bool from_key = false);
+cudaError_t launch_verlet_flag(sph_handle* h, cudaStream_t st);
 // gate (Verlet mode): device flag, the mesh kernels return at once while gate[0] == 0
 cudaError_t launch_build_grid(sph_handle* h, const sph_state& s, cudaStream_t st, const int* gate = nullptr);
-cudaError_t launch_verlet_flag(sph_handle* h, cudaStream_t st);
 // eorder: write the packs in the unit-major evaluation order of the last build (e_of_c), the
 // particle of each evaluation slot (perm_e) and, at builds, the cell-order copy packAc
-// list_counters: also zero the counters of the list build and list evaluation
-// that follow in the step (which then need no memsets of their own)
+// Also zeroes the work counters of the pair kernels that follow, which need no memsets
+// of their own, and, unless keep_counts (reverse mode), the pair counts
 cudaError_t launch_pack(sph_handle* h, const sph_state& s, bool predict, cudaStream_t st, bool eorder = false,
-                        bool list_counters = false);
-// next_dt: also leave the CFL block minima of the new state in h->part (the next
-// step's dt without a k_derive pass)
+                        bool keep_counts = false);
+// next_dt: also leave the CFL keys of the new state in dt_key (the next step's
+// dt without a k_cfl pass)
 cudaError_t launch_kick2(sph_handle* h, const sph_state& s, double* t_dev, cudaStream_t st, bool next_dt = false);
 // order: the particle to place at each position (NULL: h->perm, the cell order of the last mesh)
 cudaError_t launch_renumber(sph_handle* h, sph_state& s, cudaStream_t st, const int32_t* order = nullptr);
@@ -464,8 +468,8 @@ cudaError_t launch_pair_vjp(sph_handle* h, const sph_state& s, const void* G, co
                             cudaStream_t st, const void* A64 = nullptr, const void* B64 = nullptr,
                             const void* C64 = nullptr);
 // Verlet lists: build (k_pair over the (1 + beta) radius, returns at once unless vflag[0]) and
-// the pair evaluation over the lists; both only after a launch_pack with list_counters in
-// the same step, which zeroes their counters
+// the pair evaluation over the lists; both only after a launch_pack in the same step, which
+// zeroes their counters
 cudaError_t launch_list_build(sph_handle* h, const sph_state& s, cudaStream_t st);
 // kick2: also the second half kick of the step (and the instance time, and with
 // next_dt the CFL keys of the new state), fused into the rate write

@@ -265,7 +265,7 @@ cudaError_t launch_list_build(sph_handle* h, const sph_state& s, cudaStream_t st
     a.e_of_c = h->e_of_c;
     a.Ac = h->packAc;
   }
-  // work counter zeroed by the step's k_pack (launch_pack with list_counters)
+  // work counter zeroed by the step's k_pack
   a.work_counter = &h->counters[7];
   a.vinst = h->n_inst > 1 ? h->vinst : nullptr;   // only the instances whose lists are rebuilt
   cudaError_t e = h->dp.precision == SPH_PREC_MIXED ? launch_dim<true>(h, a, st) : launch_dim<false>(h, a, st);

@@ -564,8 +564,16 @@ cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st)
   while (a.group > 8 && a.n < (int64_t)4 * sms * a.group) a.group >>= 1;
   const int64_t groups = (a.n + a.group - 1) / a.group;
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
-  const int grid = groups < (int64_t)sms * b ? (int)groups : sms * b;
-  return launch_chained(k_pair<MIXED, DIM, MODE, HLL, EXTRA>, dim3(grid), dim3(kPairBlock), st, a);
+  // few groups: one CTA per SM until each holds a group per warp (a CTA's warps
+  // sit on the SM's four schedulers in turn), then as many CTAs as that needs
+  const int64_t want = groups < sms ? groups : ((groups + kWarps - 1) / kWarps > sms ? (groups + kWarps - 1) / kWarps : sms);
+  const int grid = want < (int64_t)sms * b ? (int)want : sms * b;
+  // A plain launch, not chained to the kernel before it: CTAs that become
+  // resident while that one still runs are packed onto the SMs with room left
+  // instead of being spread over all of them (6k particles in a plane, FP64, a
+  // step: 0.30 ms spread, 0.38 ms packed).
+  k_pair<MIXED, DIM, MODE, HLL, EXTRA><<<grid, kPairBlock, 0, st>>>(a);
+  return cudaGetLastError();
 }
 
 template <bool MIXED, int MODE, bool HLL, bool EXTRA>
@@ -615,28 +623,23 @@ cudaError_t launch_pair_vjp(sph_handle* h, const sph_state& s, const void* G, co
     a.C = C64;
     a.vinv = 1.0;
   }
-  cudaError_t e = cudaMemsetAsync(&h->counters[5], 0, sizeof(unsigned long long), st);
-  if (e != cudaSuccess) return e;
-  e = fp64 ? launch_dim<false, kModeVjp>(h, a, st) : launch_dim<true, kModeVjp>(h, a, st);
+  const cudaError_t e = fp64 ? launch_dim<false, kModeVjp>(h, a, st) : launch_dim<true, kModeVjp>(h, a, st);
   h->launches += 1;
   return e;
 }
 
 cudaError_t launch_pair(sph_handle* h, const sph_state& s, cudaStream_t st) {
   PairArgs a = make_args(h, s);
-  cudaError_t e = cudaMemsetAsync(h->counters, 0, 3 * sizeof(unsigned long long), st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(&h->counters[4], 0, 2 * sizeof(unsigned long long), st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;   // counters zeroed by the k_pack before
   if (h->order2) {
     // SPH gradients first (their own pass over the same pair set), then the rates
     a.gP = h->grad_p;
     a.gV = h->grad_v;
-    e = h->dp.precision == SPH_PREC_MIXED ? launch_dim<true, kModeGrad>(h, a, st)
-                                          : launch_dim<false, kModeGrad>(h, a, st);
+    PairArgs ag = a;
+    ag.work_counter = &h->counters[7];
+    e = h->dp.precision == SPH_PREC_MIXED ? launch_dim<true, kModeGrad>(h, ag, st)
+                                          : launch_dim<false, kModeGrad>(h, ag, st);
     h->launches += 1;
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(&h->counters[5], 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
   }
   if ((e = prof_record(h, true, st)) != cudaSuccess) return e;

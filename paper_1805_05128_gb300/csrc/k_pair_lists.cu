@@ -555,7 +555,7 @@ cudaError_t launch_pair_lists(sph_handle* h, const sph_state& s, cudaStream_t st
   a.kx_t = t_dev;
   a.dt_key = h->dt_key;
   a.dp = h->dp;
-  // pair counts and work counter zeroed by the step's k_pack (launch_pack with list_counters)
+  // pair counts and work counter zeroed by the step's k_pack
   cudaError_t e = cudaSuccess;
   if (h->unit_sched != SPH_SCHED_GLOBAL) {
     // operands, lists and rows in the unit-major evaluation order; per-unit

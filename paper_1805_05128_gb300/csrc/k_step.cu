@@ -41,13 +41,13 @@ __device__ __forceinline__ int fkey(float x) {
 __device__ __forceinline__ float funkey(int k) { return __int_as_float(k < 0 ? k ^ 0x7fffffff : k); }
 
 struct Red {
-  long long lo[3], hi[3], d1, d2, dtmin, viol;
+  long long lo[3], hi[3], d1, d2, viol;
   int dlo[3], dhi[3];
 };
 
 __device__ __forceinline__ void red_init(Red& r) {
   for (int a = 0; a < 3; ++a) { r.lo[a] = LLONG_MAX; r.hi[a] = LLONG_MIN; r.dlo[a] = INT_MAX; r.dhi[a] = INT_MIN; }
-  r.d1 = 0; r.d2 = 0; r.dtmin = LLONG_MAX; r.viol = LLONG_MIN;
+  r.d1 = 0; r.d2 = 0; r.viol = LLONG_MIN;
 }
 
 __device__ __forceinline__ void red_merge(Red& a, const Red& b) {
@@ -58,7 +58,6 @@ __device__ __forceinline__ void red_merge(Red& a, const Red& b) {
     a.dhi[k] = max(a.dhi[k], b.dhi[k]);
   }
   top2_merge(a.d1, a.d2, b.d1, b.d2);
-  a.dtmin = a.dtmin < b.dtmin ? a.dtmin : b.dtmin;
   a.viol = a.viol > b.viol ? a.viol : b.viol;
 }
 
@@ -72,7 +71,6 @@ __device__ __forceinline__ Red shfl_red(const Red& r, int o) {
   }
   q.d1 = __shfl_xor_sync(0xffffffffu, r.d1, o);
   q.d2 = __shfl_xor_sync(0xffffffffu, r.d2, o);
-  q.dtmin = __shfl_xor_sync(0xffffffffu, r.dtmin, o);
   q.viol = __shfl_xor_sync(0xffffffffu, r.viol, o);
   return q;
 }
@@ -89,6 +87,7 @@ __device__ void block_reduce(Red& r) {
   __syncthreads();
   if (t == 0)
     for (int w = 1; w < kBlock / 32; ++w) red_merge(r, sh[w]);
+  __syncthreads();
 }
 
 // Block minimum of the dt keys only (a step's k_derive); result in thread 0.
@@ -109,27 +108,21 @@ __device__ long long block_min_key(long long k) {
 __device__ __forceinline__ void write_part(BlockPart* part, const Red& r) {
   BlockPart& b = part[blockIdx.x];
   for (int a = 0; a < 3; ++a) { b.lo[a] = r.lo[a]; b.hi[a] = r.hi[a]; }
-  b.d1 = r.d1; b.d2 = r.d2; b.dtmin = r.dtmin;
+  b.d1 = r.d1; b.d2 = r.d2;
 }
 
 // ---------------------------------------------------------------------------
-// d, P, c at the current state, dt_i = eta d_i / (c_i + |v_i|) (cfl_key),
-// optional bbox.
+// d, P, c and the bounding box of the current state (a mesh build outside the
+// step follows), or a step's CFL bound dt_i = eta d_i / (c_i + |v_i|)
+// (cfl_key), min-reduced into the instance's dt_key.
 // ---------------------------------------------------------------------------
 __global__ void k_derive(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
-                         const int64_t* __restrict__ blk_end, BlockPart* part, int write_derived,
-                         int with_bbox) {
+                         const int64_t* __restrict__ blk_end, BlockPart* part) {
   chain_entry();
   int64_t p = blk_start[blockIdx.x] + threadIdx.x;
   Red r;
   red_init(r);
-  if (p < blk_end[blockIdx.x] && !with_bbox && !write_derived) {
-    // a step's CFL bound only (every load issued before the arithmetic)
-    const double vx = ld(s.vx, p), vy = ld(s.vy, p), vz = ld(s.vz, p);
-    const double E = s.E[p], rho = s.rho[p], m = s.m[p];
-    const int mi = s.mat ? s.mat[p] : 0;
-    r.dtmin = cfl_key(P, vx, vy, vz, E, rho, m, mi);
-  } else if (p < blk_end[blockIdx.x]) {
+  if (p < blk_end[blockIdx.x]) {
     double vx = ld(s.vx, p), vy = ld(s.vy, p), vz = ld(s.vz, p);
     double v2 = vx * vx + vy * vy + vz * vz;
     double e = s.E[p] - 0.5 * v2;
@@ -137,72 +130,70 @@ __global__ void k_derive(DevParams P, sph_state s, const int64_t* __restrict__ b
     double Pp, cp;
     eos(P.mat[mi], s.rho[p], e, Pp, cp);
     double d = size_of(P.dim, s.m[p], s.rho[p]);
-    if (write_derived) { s.d[p] = d; s.P[p] = Pp; s.c[p] = cp; }
-    r.dtmin = dkey((P.eta * d) / (cp + sqrt(v2)));
-    if (with_bbox) {
-      r.lo[0] = r.hi[0] = dkey(s.x[p]);
-      if (P.dim >= 2) r.lo[1] = r.hi[1] = dkey(s.y[p]);
-      if (P.dim >= 3) r.lo[2] = r.hi[2] = dkey(s.z[p]);
-      r.d1 = dkey(d);
-    }
-  }
-  if (!with_bbox) {   // a step's dt: only the minimum is read (the other partials come from k_kick_drift)
-    const long long k = block_min_key(r.dtmin);
-    if (threadIdx.x == 0) part[blockIdx.x].dtmin = k;
-    return;
+    s.d[p] = d; s.P[p] = Pp; s.c[p] = cp;
+    r.lo[0] = r.hi[0] = dkey(s.x[p]);
+    if (P.dim >= 2) r.lo[1] = r.hi[1] = dkey(s.y[p]);
+    if (P.dim >= 3) r.lo[2] = r.hi[2] = dkey(s.z[p]);
+    r.d1 = dkey(d);
   }
   block_reduce(r);
   if (threadIdx.x == 0) write_part(part, r);
 }
 
-// One block per instance: the step's dt = cfl * (minimum of the instance's
-// block minima).  Only the dtmin fields are read, four independent loads in
-// flight per thread.
-__global__ void k_reduce_dt(const int32_t* __restrict__ inst_blk, const BlockPart* __restrict__ part, double cfl,
-                            double* dt, long long* dt_key, int from_key) {
+__global__ void k_cfl(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
+                      const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst, long long* dt_key) {
   chain_entry();
-  const int b = blockIdx.x;
-  if (from_key) {   // the fused second kick's keys: already the instance minimum
-    if (threadIdx.x == 0) {
-      dt[b] = cfl * dunkey(dt_key[b]);
-      dt_key[b] = LLONG_MAX;
-    }
-    return;
+  const int64_t p = blk_start[blockIdx.x] + threadIdx.x;
+  long long k = LLONG_MAX;
+  if (p < blk_end[blockIdx.x]) {
+    // every load issued before the arithmetic
+    const double vx = ld(s.vx, p), vy = ld(s.vy, p), vz = ld(s.vz, p);
+    const double E = s.E[p], rho = s.rho[p], m = s.m[p];
+    const int mi = s.mat ? s.mat[p] : 0;
+    k = cfl_key(P, vx, vy, vz, E, rho, m, mi);
   }
-  const int k0 = inst_blk[b], k1 = inst_blk[b + 1];
-  long long m = LLONG_MAX;
-  for (int k = k0 + threadIdx.x; k < k1; k += 4 * blockDim.x) {
-    long long q[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int kk = k + u * blockDim.x;
-      q[u] = kk < k1 ? part[kk].dtmin : LLONG_MAX;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) m = q[u] < m ? q[u] : m;
-  }
-  m = block_min_key(m);
-  if (threadIdx.x == 0) {
-    dt[b] = cfl * dunkey(m);
-    dt_key[b] = LLONG_MAX;   // the next accumulation starts afresh
-  }
+  k = block_min_key(k);
+  if (threadIdx.x == 0) atomicMin(&dt_key[blk_inst[blockIdx.x]], k);
 }
+
+// dt = cfl * (the instance's minimum), and the keys ready for the next
+// accumulation (sph_cfl_dt; a step's kick-drift forms its own dt).
+__global__ void k_reduce_dt(int n_inst, double cfl, double* dt, long long* dt_key) {
+  chain_entry();
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= n_inst) return;
+  dt[b] = cfl * dunkey(dt_key[b]);
+  dt_key[b] = LLONG_MAX;
+}
+
+// Arguments of the mesh build.
+struct MeshArgs {
+  DevParams P;
+  const double *x, *y, *z;
+  int n_inst, nblk;
+  const int64_t *inst_off, *inst_cap, *blk_start, *blk_end;
+  const int32_t *blk_inst, *inst_blk;
+  const BlockPart* part;
+  GridInfo* grid;
+  int64_t* total_cells;
+  int32_t *cell_count, *cell_start, *scan_sums, *cell_of, *rank, *perm;
+  double* slot_org;         // mixed precision: origin of each slot's cell, or NULL
+  int* status;
+  const int* gate;          // Verlet steps: nothing is built while gate[0] == 0
+  const int* vinst;         // Verlet steps of a batched handle: the instances rebuilt, or NULL (all)
+};
 
 // One block per instance: the bounding box and the two largest sizes of the
 // instance from its block partials, into the grid record.
 // vinst (Verlet steps): an instance that keeps its lists keeps its mesh geometry.
-__global__ void k_reduce_inst(const int32_t* __restrict__ inst_blk, const BlockPart* __restrict__ part,
-                              GridInfo* grid, const int* __restrict__ gate, const int* __restrict__ vinst) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
-  int b = blockIdx.x;
+__device__ void mesh_reduce_inst(int b, const int32_t* inst_blk, const BlockPart* part, GridInfo* grid, const int* vinst) {
   if (vinst && vinst[b] == 0) return;
   Red r;
   red_init(r);
   for (int k = inst_blk[b] + threadIdx.x; k < inst_blk[b + 1]; k += blockDim.x) {
     Red q;
     for (int a = 0; a < 3; ++a) { q.lo[a] = part[k].lo[a]; q.hi[a] = part[k].hi[a]; }
-    q.d1 = part[k].d1; q.d2 = part[k].d2; q.dtmin = part[k].dtmin;
+    q.d1 = part[k].d1; q.d2 = part[k].d2;
     red_merge(r, q);
   }
   block_reduce(r);
@@ -220,11 +211,8 @@ __global__ void k_reduce_inst(const int32_t* __restrict__ inst_blk, const BlockP
 // in instance order.  Matches the oracle bit for bit.
 // vinst (Verlet steps): an instance that keeps its lists keeps its geometry and
 // only moves to its new cell offset.
-__global__ void k_grid_setup(DevParams P, int n_inst, const int64_t* __restrict__ inst_off,
-                             const int64_t* __restrict__ inst_cap, GridInfo* grid, int64_t* total_cells,
-                             int* status, const int* __restrict__ gate, const int* __restrict__ vinst) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
+__device__ void mesh_setup(const DevParams& P, int n_inst, const int64_t* inst_off, const int64_t* inst_cap, GridInfo* grid,
+                           int64_t* total_cells, int* status, const int* vinst) {
   // the instances' meshes, one thread per instance
   for (int b = threadIdx.x; b < n_inst; b += blockDim.x) {
     GridInfo& g = grid[b];
@@ -302,38 +290,32 @@ __device__ __forceinline__ int64_t local_cell(const GridInfo& g, int dim, double
   return (int64_t)c[0] + (int64_t)g.dims[0] * ((int64_t)c[1] + (int64_t)g.dims[1] * c[2]);
 }
 
+// One segmented block's particles (t: the thread's position in the block).
 // vinst (Verlet steps): the particles of an instance that keeps its lists are
 // counted at their positions of its last build (vref), with its kept
 // geometry, which reproduces that build's cells, slots and in-cell order.
-__global__ void k_cell_count(int dim, sph_state s, const int64_t* __restrict__ blk_start,
-                             const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst, int nblk,
-                             const GridInfo* __restrict__ grid, int32_t* cell_count, int32_t* cell_of,
-                             int32_t* rank, int* status, const int* __restrict__ gate, const int* __restrict__ vinst,
-                             const double* __restrict__ vref, int64_t n) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
-  // a capped grid strides over the segmented blocks (cheap to launch when gated)
-  for (int lb = blockIdx.x; lb < nblk; lb += gridDim.x) {
-    const int64_t p = blk_start[lb] + threadIdx.x;
-    if (p >= blk_end[lb]) continue;
-    const int b = blk_inst[lb];
-    const GridInfo& g = grid[b];
-    const bool kept = vinst && vinst[b] == 0;
-    const double px = kept ? vref[p] : s.x[p];
-    const double py = dim >= 2 ? (kept ? vref[n + p] : s.y[p]) : 0.0;
-    const double pz = dim >= 3 ? (kept ? vref[2 * n + p] : s.z[p]) : 0.0;
-    int32_t c[3];
-    int64_t lc = local_cell(g, dim, px, py, pz, c);
-    bool ok = true;
-    for (int a = 0; a < 3; ++a) ok = ok && c[a] >= 0 && c[a] < g.dims[a];
-    if (!ok) {  // only a non-finite position can leave the mesh: latch it, stay in bounds
-      set_status(status, SPH_ERR_NONFINITE);
-      lc = 0;
-    }
-    const int32_t gc = (int32_t)(g.cell_off + lc);
-    cell_of[p] = gc;
-    rank[p] = atomicAdd(&cell_count[gc], 1);
+__device__ __forceinline__ void mesh_count(const MeshArgs& a, int lb, int t) {
+  const int dim = a.P.dim;
+  const int64_t p = a.blk_start[lb] + t;
+  if (p >= a.blk_end[lb]) return;
+  const int b = a.blk_inst[lb];
+  const GridInfo& g = a.grid[b];
+  const bool kept = a.vinst && a.vinst[b] == 0;
+  const double* vref = a.P.vref;
+  const double px = kept ? vref[p] : a.x[p];
+  const double py = dim >= 2 ? (kept ? vref[a.P.n + p] : a.y[p]) : 0.0;
+  const double pz = dim >= 3 ? (kept ? vref[2 * a.P.n + p] : a.z[p]) : 0.0;
+  int32_t c[3];
+  int64_t lc = local_cell(g, dim, px, py, pz, c);
+  bool ok = true;
+  for (int k = 0; k < 3; ++k) ok = ok && c[k] >= 0 && c[k] < g.dims[k];
+  if (!ok) {  // only a non-finite position can leave the mesh: latch it, stay in bounds
+    set_status(a.status, SPH_ERR_NONFINITE);
+    lc = 0;
   }
+  const int32_t gc = (int32_t)(g.cell_off + lc);
+  a.cell_of[p] = gc;
+  a.rank[p] = atomicAdd(&a.cell_count[gc], 1);
 }
 
 // Exclusive scan of cell_count[0, total) into cell_start, 1024 cells per tile.
@@ -434,43 +416,38 @@ __global__ void k_scan_down(int32_t* cnt, const int64_t* __restrict__ total, con
 // vinst (Verlet steps): the slots of an instance that keeps its lists keep
 // their particles (its cells' starts come out as before), so its particles
 // are not scattered, and its cells are not sorted below.
-__global__ void k_cell_scatter(int64_t n, const int32_t* __restrict__ cell_of, const int32_t* __restrict__ rank,
-                               const int32_t* __restrict__ start, int32_t* perm, const int* __restrict__ gate,
-                               const int* __restrict__ vinst, const int64_t* __restrict__ inst_off, int n_inst) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
-  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-    if (vinst) {
-      int lo = 0, hi = n_inst;                       // the particle's instance
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (inst_off[mid] <= p) lo = mid; else hi = mid;
-      }
-      if (vinst[lo] == 0) continue;
+__device__ __forceinline__ void mesh_scatter(const MeshArgs& a, int64_t p) {
+  if (a.vinst) {
+    int lo = 0, hi = a.n_inst;                       // the particle's instance
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (a.inst_off[mid] <= p) lo = mid; else hi = mid;
     }
-    perm[start[cell_of[p]] + rank[p]] = (int32_t)p;
+    if (a.vinst[lo] == 0) return;
   }
+  a.perm[a.cell_start[a.cell_of[p]] + a.rank[p]] = (int32_t)p;
 }
 
 // Within each cell, order the particles by index (the atomic arrival order is
 // not reproducible; this makes the slot order a function of the state only).
 // Mixed precision: also the origin of each cell, o = x0 + c dc per axis, for
 // every slot of the cell (slot_org; k_pack takes the FP32 offsets from it).
-__global__ void k_cell_sort(const int64_t* __restrict__ total, const int32_t* __restrict__ start, int32_t* perm,
-                            const int* __restrict__ gate, const GridInfo* __restrict__ grid, int n_inst, int dim,
-                            int64_t nslots, double* slot_org, const int* __restrict__ vinst) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
+// w0, nw: this warp's index and the number of warps.
+__device__ __forceinline__ void mesh_sort(const MeshArgs& a, int64_t tot, int64_t w0, int64_t nw) {
+  const int32_t* start = a.cell_start;
+  int32_t* perm = a.perm;
+  const GridInfo* grid = a.grid;
+  const int n_inst = a.n_inst, dim = a.P.dim;
+  const int64_t nslots = a.P.n;
+  double* slot_org = a.slot_org;
+  const int* vinst = a.vinst;
   // One warp per cell: each lane holds up to kSortPer of the cell's particle
   // indices and counts, by broadcasts, the cell's indices smaller than each
   // (indices are distinct), which is its position in ascending order.  Cells
   // above 32 kSortPer particles (never on a sane mesh: the cell code admits
   // 2047) are sorted by one lane.
   constexpr int kSortPer = 4;
-  const int64_t tot = *total;
   const int lane = threadIdx.x & 31;
-  const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t c = w0; c < tot; c += nw) {
     const int b = start[c], e = start[c + 1], n = e - b;
     if (n <= 0) continue;
@@ -535,20 +512,117 @@ __global__ void k_cell_sort(const int64_t* __restrict__ total, const int32_t* __
 }
 
 // ---------------------------------------------------------------------------
+// The mesh build, a kernel per phase, chained (a chained launch that returns at
+// once costs 1.5 us).  One kernel for all phases was measured and dropped: with
+// a barrier over a cooperative grid a build of 6k particles took 84 us longer,
+// with one cluster of 16 CTAs 12 us (30 us at 32k, whose work 16 SMs hold too
+// long); the gated steps gained 2 us.
+// ---------------------------------------------------------------------------
+__global__ void k_mesh_reduce(MeshArgs a) {
+  chain_entry();
+  if (a.gate && a.gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
+  mesh_reduce_inst(blockIdx.x, a.inst_blk, a.part, a.grid, a.vinst);
+}
+
+__global__ void k_mesh_setup(MeshArgs a) {
+  chain_entry();
+  if (a.gate && a.gate[0] == 0) return;
+  if (a.n_inst == 1) {                    // one instance: no launch of its own for the reduction
+    mesh_reduce_inst(0, a.inst_blk, a.part, a.grid, a.vinst);
+    __syncthreads();
+  }
+  mesh_setup(a.P, a.n_inst, a.inst_off, a.inst_cap, a.grid, a.total_cells, a.status, a.vinst);
+}
+
+__global__ void k_cell_count(MeshArgs a) {
+  chain_entry();
+  if (a.gate && a.gate[0] == 0) return;
+  // a capped grid strides over the segmented blocks (cheap to launch when gated)
+  for (int lb = blockIdx.x; lb < a.nblk; lb += gridDim.x) mesh_count(a, lb, threadIdx.x);
+}
+
+__global__ void k_cell_scatter(MeshArgs a) {
+  chain_entry();
+  if (a.gate && a.gate[0] == 0) return;
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.P.n; p += (int64_t)gridDim.x * blockDim.x)
+    mesh_scatter(a, p);
+}
+
+__global__ void k_cell_sort(MeshArgs a) {
+  chain_entry();
+  if (a.gate && a.gate[0] == 0) return;
+  mesh_sort(a, *a.total_cells, ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+            ((int64_t)gridDim.x * blockDim.x) >> 5);
+}
+
+// Verlet lists: vflag[0] = lists invalid (vflag[1]) or the validity criterion
+// of k_kick_drift failed for some particle of any instance.
+// Also sets, per instance (no pair joins two instances), the frame
+// displacement U of the next step's criterion: the midpoint of this step's
+// displacement box, which covers k steps since the build, extrapolated to
+// k + 1 steps; after a build, one step's worth of it (the new reference is
+// this step's state); 0 while the reference is void.  Any U keeps the
+// criterion sound; a good one only makes builds rarer.
+__global__ void k_verlet_flag(int* vflag, double* vframe, VAcc* vacc, int n_inst, int* vinst, int together) {
+  chain_entry();
+  // each instance whose criterion failed is rebuilt (its mesh, slots and lists;
+  // the other instances keep theirs), or all of them when the lists are void or
+  // the instances share an evaluation order (together)
+  int fail = 0;
+  for (int b = threadIdx.x; b < n_inst; b += blockDim.x) fail |= vacc[b].viol > 0 ? 1 : 0;
+  const bool void_ref = vflag[1] != 0;
+  const bool any = __syncthreads_or(fail) != 0 || void_ref;
+  if (threadIdx.x == 0) vflag[0] = any ? 1 : 0;
+  for (int b = threadIdx.x; b < n_inst; b += blockDim.x) {
+    const bool rebuild = void_ref || (together ? any : vacc[b].viol > 0);
+    vinst[b] = rebuild ? 1 : 0;
+    VAcc& va = vacc[b];
+    int bx[6];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) { bx[a] = va.dlo[a]; bx[3 + a] = va.dhi[a]; }
+    // reset for the next kick-drift
+    va.viol = LLONG_MIN;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) { va.dlo[a] = INT_MAX; va.dhi[a] = INT_MIN; }
+    double* fr = vframe + 6 * b;
+    const double ks = fr[3] >= 1.0 ? fr[3] : 1.0;   // steps covered by this step's displacements
+    float* Uf = reinterpret_cast<float*>(fr + 4);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      // midpoint of the box of x - x^b, from that of x - x^b - U
+      const double mid = bx[a] <= bx[3 + a] ? 0.5 * ((double)funkey(bx[a]) + (double)funkey(bx[3 + a])) + fr[a]
+                                            : fr[a];
+      fr[a] = void_ref ? 0.0 : (rebuild ? mid / ks : mid * (ks + 1.0) / ks);
+      Uf[a] = (float)fr[a];
+    }
+    fr[3] = rebuild ? 1.0 : ks + 1.0;
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Kick-drift: v <- v + dt/2 a, x <- x + dt v, rho, E half kicks; predicted
 // size d~ from rho~ = rho^h + dt/2 drho; bounding box and sizes for the mesh.
 // ---------------------------------------------------------------------------
+// The time step: with dt_key, cfl times the instance's minimum, which the
+// instance's first block also leaves in dt (k_pack makes the key ready for the
+// next accumulation); else the prescribed dt.
+// (The rebuild decision of a Verlet step stays a kernel of its own: made by the
+// last block of this one, the fence and the ticket of every block added 16 us
+// at 1.125M particles, four times that kernel.)
 template <bool MIXED>
 __global__ void __launch_bounds__(kBlock, 4) k_kick_drift(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
                              const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst,
-                             const double* __restrict__ dt, BlockPart* part, int* status) {
+                             const int32_t* __restrict__ inst_blk, double* dt, const long long* __restrict__ dt_key,
+                             BlockPart* part, int* status) {
   chain_entry();
   int64_t p = blk_start[blockIdx.x] + threadIdx.x;
   Red r;
   red_init(r);
+  const int inst = blk_inst[blockIdx.x];
+  if (dt_key && threadIdx.x == 0 && inst_blk[inst] == (int)blockIdx.x) dt[inst] = P.cfl * dunkey(dt_key[inst]);
   if (p < blk_end[blockIdx.x]) {
     const int dim = P.dim;
-    const double h = dt[blk_inst[blockIdx.x]];
+    const double h = dt_key ? P.cfl * dunkey(dt_key[inst]) : dt[inst];
     const double hdt = 0.5 * h;
     double* X[3] = {s.x, s.y, s.z};
     double* V[3] = {s.vx, s.vy, s.vz};
@@ -598,7 +672,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_kick_drift(DevParams P, sph_state
       // the bound itself in FP32: the 5 % margin dwarfs its rounding).
       // (The displacement and U in FP32: their rounding, ~1e-7 of each, is far
       // inside the margin.)  The box is that of x - x^b - U.
-      const float* Uf = reinterpret_cast<const float*>(P.vframe + 6 * blk_inst[blockIdx.x] + 4);
+      const float* Uf = reinterpret_cast<const float*>(P.vframe + 6 * inst + 4);
       float dsq = 0.0f;
 #pragma unroll
       for (int a = 0; a < 3; ++a)
@@ -617,7 +691,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_kick_drift(DevParams P, sph_state
   if (threadIdx.x == 0) {
     write_part(part, r);
     if (P.vacc) {                  // the criterion's maximum and displacement box of the instance
-      VAcc* va = P.vacc + blk_inst[blockIdx.x];
+      VAcc* va = P.vacc + inst;
       atomicMax(&va->viol, r.viol);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -629,13 +703,13 @@ __global__ void __launch_bounds__(kBlock, 4) k_kick_drift(DevParams P, sph_state
 }
 
 // Second half kick with the rates of the predicted state; instance time.
-// With part, also the block minima of the CFL keys at the new state, which
-// the next step of the same sph_step call takes instead of a k_derive pass.
+// With dt_key, also the instance's minimum of the CFL keys at the new state,
+// which the next step of the same sph_step call takes instead of a k_cfl pass.
 template <bool MIXED>
 __global__ void k_kick2(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
                         const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst,
                         const int32_t* __restrict__ inst_blk, const double* __restrict__ dt, double* t_dev,
-                        BlockPart* part) {
+                        long long* dt_key) {
   chain_entry();
   const int64_t p = blk_start[blockIdx.x] + threadIdx.x;
   const int b = blk_inst[blockIdx.x];
@@ -653,7 +727,7 @@ __global__ void k_kick2(DevParams P, sph_state s, const int64_t* __restrict__ bl
     const double rho0 = s.rho[p], drho = s.drho[p], E0 = s.E[p], dE = s.dE[p];
     double m = 0.0;
     int mi = 0;
-    if (part) { m = s.m[p]; mi = s.mat ? s.mat[p] : 0; }
+    if (dt_key) { m = s.m[p]; mi = s.mat ? s.mat[p] : 0; }
 #pragma unroll
     for (int a = 0; a < 3; ++a)
       if (a < dim) v[a] = axpy<MIXED>(hdt, acc[a], v[a]);
@@ -664,11 +738,11 @@ __global__ void k_kick2(DevParams P, sph_state s, const int64_t* __restrict__ bl
       if (a < dim) V[a][p] = v[a];
     s.rho[p] = rho;
     s.E[p] = E;
-    if (part) key = cfl_key(P, v[0], v[1], v[2], E, rho, m, mi);
+    if (dt_key) key = cfl_key(P, v[0], v[1], v[2], E, rho, m, mi);
   }
-  if (part) {   // uniform over the grid: every thread reaches the block barrier
+  if (dt_key) {   // uniform over the grid: every thread reaches the block barrier
     const long long k = block_min_key(key);
-    if (threadIdx.x == 0) part[blockIdx.x].dtmin = k;
+    if (threadIdx.x == 0) atomicMin(&dt_key[b], k);
   }
 }
 
@@ -690,17 +764,23 @@ __global__ void __launch_bounds__(kBlock, 4) k_pack(DevParams P, sph_state s, co
                        void* packA, void* packB, void* packC, double* rho_slot, int32_t* slot_cell,
                        int32_t* slot_unit, int n_units, int* status, const int32_t* __restrict__ e_of_c,
                        int32_t* perm_e, void* packAc, const int* __restrict__ gate,
-                       unsigned long long* list_counters) {
+                       unsigned long long* counters, int keep_counts, const int32_t* __restrict__ inst_blk,
+                       long long* dt_key) {
   chain_entry();
-  // the counters of the list build and the list evaluation that follow (the
-  // evaluation's pair counts and work counter, the build's work counter)
-  if (list_counters && blockIdx.x == 0 && threadIdx.x == 0) {
-    list_counters[0] = 0ull;
-    list_counters[1] = 0ull;
-    list_counters[2] = 0ull;
-    list_counters[5] = 0ull;
-    list_counters[7] = 0ull;
+  // the counters of the pair kernels that follow: the evaluation's pair counts
+  // (kept by the reverse mode) and the work counters
+  if (counters && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (!keep_counts) {
+      counters[0] = 0ull;
+      counters[1] = 0ull;
+      counters[2] = 0ull;
+      counters[4] = 0ull;
+    }
+    counters[5] = 0ull;
+    counters[7] = 0ull;
   }
+  // the CFL keys, read by the kick-drift, are ready for the next accumulation
+  if (dt_key && threadIdx.x == 0 && inst_blk[blk_inst[blockIdx.x]] == (int)blockIdx.x) dt_key[blk_inst[blockIdx.x]] = LLONG_MAX;
   const int64_t sc = blk_start[blockIdx.x] + threadIdx.x;     // cell-order slot
   if (sc >= blk_end[blockIdx.x]) return;
   // the operands go to the slot's evaluation position (unit-major order of the
@@ -883,99 +963,34 @@ static int capped_grid(int want) {
   return want < cap ? (want > 0 ? want : 1) : cap;
 }
 
-cudaError_t launch_derive_dt(sph_handle* h, const sph_state& s, bool with_bbox, cudaStream_t st) {
-  CKL(launch_chained(k_derive, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->part, with_bbox ? 1 : 0,
-                                       with_bbox ? 1 : 0));
+cudaError_t launch_derive(sph_handle* h, const sph_state& s, cudaStream_t st) {
+  CKL(launch_chained(k_derive, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->part));
   h->launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce_dt(sph_handle* h, cudaStream_t st, bool from_key) {
-  CKL(launch_chained(k_reduce_dt, dim3(h->n_inst), dim3(kBlock), st, h->inst_blk, h->part, h->dp.cfl, h->dt, h->dt_key, from_key ? 1 : 0));
+cudaError_t launch_cfl(sph_handle* h, const sph_state& s, cudaStream_t st) {
+  CKL(launch_chained(k_cfl, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->dt_key));
   h->launches += 1;
   return cudaGetLastError();
 }
 
-cudaError_t launch_kick_drift(sph_handle* h, const sph_state& s, cudaStream_t st) {
+cudaError_t launch_reduce_dt(sph_handle* h, cudaStream_t st) {
+  CKL(launch_chained(k_reduce_dt, dim3(grid_for(h->n_inst, kBlock)), dim3(kBlock), st, h->n_inst, h->dp.cfl, h->dt, h->dt_key));
+  h->launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t launch_kick_drift(sph_handle* h, const sph_state& s, cudaStream_t st, bool from_key) {
+  const long long* key = from_key ? h->dt_key : nullptr;
   if (h->dp.precision == SPH_PREC_MIXED)
-    CKL(launch_chained(k_kick_drift<true>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->dt, h->part,
-                                                   h->status));
+    CKL(launch_chained(k_kick_drift<true>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst,
+                       h->inst_blk, h->dt, key, h->part, h->status));
   else
-    CKL(launch_chained(k_kick_drift<false>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->dt, h->part,
-                                                    h->status));
+    CKL(launch_chained(k_kick_drift<false>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst,
+                       h->inst_blk, h->dt, key, h->part, h->status));
   h->launches += 1;
   return cudaGetLastError();
-}
-
-// Mesh from the block partials left by k_derive(with_bbox) or k_kick_drift,
-// then the counting sort of particles into cells.
-cudaError_t launch_build_grid(sph_handle* h, const sph_state& s, cudaStream_t st, const int* gate) {
-  // per-instance rebuilds only inside the Verlet sequence (gated) of a batched
-  // handle; any other build is global (one instance: the same thing)
-  const int* vinst = gate && h->n_inst > 1 ? h->vinst : nullptr;
-  CKL(launch_chained(k_reduce_inst, dim3(h->n_inst), dim3(kBlock), st, h->inst_blk, h->part, h->grid, gate, vinst));
-  CKL(launch_chained(k_grid_setup, dim3(1), dim3(h->n_inst < 1024 ? 32 * ((h->n_inst + 31) / 32) : 1024), st,
-                     h->dp, h->n_inst, h->inst_off, h->inst_cap, h->grid, h->total_cells, h->status, gate, vinst));
-  CKL(launch_chained(k_cell_count, dim3(capped_grid(h->nblk)), dim3(kBlock), st, h->dp.dim, s, h->blk_start,
-                     h->blk_end, h->blk_inst, h->nblk, h->grid, h->cell_count, h->cell_of, h->rank, h->status, gate,
-                     vinst, (const double*)h->vref, h->n));
-  int tiles = capped_grid(grid_for(h->cell_cap, kScanTile));
-  CKL(launch_chained(k_scan_reduce, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, gate));
-  CKL(launch_chained(k_scan_sums, dim3(1), dim3(1024), st, h->scan_sums, h->total_cells, gate));
-  CKL(launch_chained(k_scan_down, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, h->cell_start, h->n, gate));
-  CKL(launch_chained(k_cell_scatter, dim3(capped_grid(grid_for(h->n, kBlock))), dim3(kBlock), st, h->n, h->cell_of,
-                     h->rank, h->cell_start, h->perm, gate, vinst, h->inst_off, h->n_inst));
-  CKL(launch_chained(k_cell_sort, dim3(capped_grid(grid_for(h->cell_cap * 32, kBlock))), dim3(kBlock), st,
-                     h->total_cells, h->cell_start, h->perm, gate, h->grid, h->n_inst, h->dp.dim, h->n, h->slot_org,
-                     vinst));
-  h->launches += 8;
-  // a mesh built outside the Verlet sequence changes the slot order under the lists
-  if (!gate && h->verlet) return cudaMemsetAsync(&h->vflag[1], 0xff, sizeof(int), st);
-  return cudaGetLastError();
-}
-
-// Verlet lists: vflag[0] = lists invalid (vflag[1]) or the validity criterion
-// of k_kick_drift failed for some particle of any instance.
-// Also sets, per instance (no pair joins two instances), the frame
-// displacement U of the next step's criterion: the midpoint of this step's
-// displacement box, which covers k steps since the build, extrapolated to
-// k + 1 steps; after a build, one step's worth of it (the new reference is
-// this step's state); 0 while the reference is void.  Any U keeps the
-// criterion sound; a good one only makes builds rarer.
-__global__ void k_verlet_flag(int* vflag, double* vframe, VAcc* vacc, int n_inst, int* vinst, int together) {
-  chain_entry();
-  // each instance whose criterion failed is rebuilt (its mesh, slots and lists;
-  // the other instances keep theirs), or all of them when the lists are void or
-  // the instances share an evaluation order (together)
-  int fail = 0;
-  for (int b = threadIdx.x; b < n_inst; b += blockDim.x) fail |= vacc[b].viol > 0 ? 1 : 0;
-  const bool void_ref = vflag[1] != 0;
-  const bool any = __syncthreads_or(fail) != 0 || void_ref;
-  if (threadIdx.x == 0) vflag[0] = any ? 1 : 0;
-  for (int b = threadIdx.x; b < n_inst; b += blockDim.x) {
-    const bool rebuild = void_ref || (together ? any : vacc[b].viol > 0);
-    vinst[b] = rebuild ? 1 : 0;
-    VAcc& va = vacc[b];
-    int bx[6];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) { bx[a] = va.dlo[a]; bx[3 + a] = va.dhi[a]; }
-    // reset for the next kick-drift
-    va.viol = LLONG_MIN;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) { va.dlo[a] = INT_MAX; va.dhi[a] = INT_MIN; }
-    double* fr = vframe + 6 * b;
-    const double ks = fr[3] >= 1.0 ? fr[3] : 1.0;   // steps covered by this step's displacements
-    float* Uf = reinterpret_cast<float*>(fr + 4);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      // midpoint of the box of x - x^b, from that of x - x^b - U
-      const double mid = bx[a] <= bx[3 + a] ? 0.5 * ((double)funkey(bx[a]) + (double)funkey(bx[3 + a])) + fr[a]
-                                            : fr[a];
-      fr[a] = void_ref ? 0.0 : (rebuild ? mid / ks : mid * (ks + 1.0) / ks);
-      Uf[a] = (float)fr[a];
-    }
-    fr[3] = rebuild ? 1.0 : ks + 1.0;
-  }
 }
 
 cudaError_t launch_verlet_flag(sph_handle* h, cudaStream_t st) {
@@ -985,9 +1000,45 @@ cudaError_t launch_verlet_flag(sph_handle* h, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// Mesh from the block partials left by k_derive or k_kick_drift, then the
+// counting sort of particles into cells.
+cudaError_t launch_build_grid(sph_handle* h, const sph_state& s, cudaStream_t st, const int* gate) {
+  MeshArgs a;
+  a.P = h->dp;
+  a.x = s.x; a.y = s.y; a.z = s.z;
+  a.n_inst = h->n_inst; a.nblk = h->nblk;
+  a.inst_off = h->inst_off; a.inst_cap = h->inst_cap; a.blk_start = h->blk_start; a.blk_end = h->blk_end;
+  a.blk_inst = h->blk_inst; a.inst_blk = h->inst_blk;
+  a.part = h->part; a.grid = h->grid; a.total_cells = h->total_cells;
+  a.cell_count = h->cell_count; a.cell_start = h->cell_start; a.scan_sums = h->scan_sums;
+  a.cell_of = h->cell_of; a.rank = h->rank; a.perm = h->perm; a.slot_org = h->slot_org;
+  a.status = h->status;
+  a.gate = gate;
+  // per-instance rebuilds only inside the Verlet sequence (gated) of a batched
+  // handle; any other build is global (one instance: the same thing)
+  a.vinst = gate && h->n_inst > 1 ? h->vinst : nullptr;
+  if (h->n_inst > 1) {
+    CKL(launch_chained(k_mesh_reduce, dim3(h->n_inst), dim3(kBlock), st, a));
+    h->launches += 1;
+  }
+  CKL(launch_chained(k_mesh_setup, dim3(1), dim3(h->n_inst == 1 ? kBlock : (h->n_inst < 1024 ? 32 * ((h->n_inst + 31) / 32) : 1024)),
+                     st, a));
+  CKL(launch_chained(k_cell_count, dim3(capped_grid(h->nblk)), dim3(kBlock), st, a));
+  int tiles = capped_grid(grid_for(h->cell_cap, kScanTile));
+  CKL(launch_chained(k_scan_reduce, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, gate));
+  CKL(launch_chained(k_scan_sums, dim3(1), dim3(1024), st, h->scan_sums, h->total_cells, gate));
+  CKL(launch_chained(k_scan_down, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, h->cell_start, h->n, gate));
+  CKL(launch_chained(k_cell_scatter, dim3(capped_grid(grid_for(h->n, kBlock))), dim3(kBlock), st, a));
+  CKL(launch_chained(k_cell_sort, dim3(capped_grid(grid_for(h->cell_cap * 32, kBlock))), dim3(kBlock), st, a));
+  h->launches += 6;
+  // a mesh built outside the Verlet sequence changes the slot order under the lists
+  if (!gate && h->verlet) return cudaMemsetAsync(&h->vflag[1], 0xff, sizeof(int), st);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_pack(sph_handle* h, const sph_state& s, bool predict, cudaStream_t st, bool eorder,
-                        bool list_counters) {
-  unsigned long long* lc = list_counters ? h->counters : nullptr;
+                        bool keep_counts) {
+  const int kc = keep_counts ? 1 : 0;
   const int32_t* eoc = eorder ? h->e_of_c : nullptr;
   int32_t* pe = eorder ? h->perm_e : nullptr;
   void* Ac = eorder ? h->packAc : nullptr;
@@ -995,12 +1046,12 @@ cudaError_t launch_pack(sph_handle* h, const sph_state& s, bool predict, cudaStr
     CKL(launch_chained(k_pack<true>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->grid, h->dt,
                                              predict ? 1 : 0, h->perm, h->cell_of, h->packA, h->packB, h->packC,
                                              h->rho_slot, h->slot_cell, h->slot_unit, h->K, h->status, eoc, pe, Ac,
-                                             h->vflag, lc));
+                                             h->vflag, h->counters, kc, h->inst_blk, h->dt_key));
   else
     CKL(launch_chained(k_pack<false>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->grid, h->dt,
                                               predict ? 1 : 0, h->perm, h->cell_of, h->packA, h->packB, h->packC,
                                               h->rho_slot, h->slot_cell, h->slot_unit, h->K, h->status, eoc, pe, Ac,
-                                              h->vflag, lc));
+                                              h->vflag, h->counters, kc, h->inst_blk, h->dt_key));
   h->launches += 1;
   return cudaGetLastError();
 }
@@ -1012,19 +1063,20 @@ cudaError_t launch_pack_fp64(sph_handle* h, const sph_state& s, bool predict, vo
                              double* rho_out, cudaStream_t st) {
   k_pack<false><<<h->nblk, kBlock, 0, st>>>(h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->grid, h->dt,
                                             predict ? 1 : 0, h->perm, h->cell_of, A, B, C, rho_out, h->slot_cell,
-                                            h->slot_unit, h->K, h->status, nullptr, nullptr, nullptr, nullptr, nullptr);
+                                            h->slot_unit, h->K, h->status, nullptr, nullptr, nullptr, nullptr, h->counters, 1,
+                                            h->inst_blk, h->dt_key);
   h->launches += 1;
   return cudaGetLastError();
 }
 
 cudaError_t launch_kick2(sph_handle* h, const sph_state& s, double* t_dev, cudaStream_t st, bool next_dt) {
-  BlockPart* part = next_dt ? h->part : nullptr;
+  long long* key = next_dt ? h->dt_key : nullptr;
   if (h->dp.precision == SPH_PREC_MIXED)
     CKL(launch_chained(k_kick2<true>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->inst_blk, h->dt,
-                                              t_dev, part));
+                                              t_dev, key));
   else
     CKL(launch_chained(k_kick2<false>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->inst_blk, h->dt,
-                                               t_dev, part));
+                                               t_dev, key));
   h->launches += 1;
   return cudaGetLastError();
 }
@@ -1082,7 +1134,7 @@ cudaError_t launch_exclusive_scan(int32_t* cnt, const int64_t* total, int32_t* s
 // (launch_exclusive_scan's three kernels are counted by its callers)
 
 cudaError_t launch_conservation(sph_handle* h, const sph_state& s, double* out, cudaStream_t st) {
-  const int per = sum_cluster_size(k_conservation, h->n / h->n_inst);
+  const int per = cluster_size_for(k_conservation, kSumBlock, h->n / h->n_inst, 4096);
   CKL(launch_clusters(k_conservation, h->n_inst, per, kSumBlock, st, s, h->inst_off, out));
   h->launches += 1;
   return cudaGetLastError();
