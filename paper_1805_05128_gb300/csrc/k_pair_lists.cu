@@ -31,6 +31,7 @@ namespace {
 // plate impact, 16 / 8 / 4 / 2 lanes per slot take 0.89 / 0.81 / 0.75 / 0.76 ms.
 constexpr int kSlotLanes = 4;
 constexpr int kSlotsPerWarp = 32 / kSlotLanes;
+constexpr int kPassCap = 256;   // FP64: list entries tested before their fluxes are evaluated
 
 // Optional staging of the neighbour operands (sph_params.list_staging): the
 // operands of the next chunk's entries are copied into shared memory with
@@ -79,6 +80,8 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
     const int c = threadIdx.x;
     unit_shift[c] = make_float4((float)(c % 3 - 1), (float)((c / 3) % 3 - 1), (float)(c / 9 - 1), 0.f);
   }
+  // FP64: the accepted entries' slots, a segment of the list at a time
+  __shared__ uint32_t passed[MIXED ? 1 : kWarps][MIXED ? 1 : kSlotsPerWarp][MIXED ? 1 : kPassCap];
   const int adj_n = EXTRA && a.collect_adj ? a.K * a.adj_words : 0;   // the block's adjacency tile
   if constexpr (EXTRA)
     for (int w = threadIdx.x; w < adj_n; w += blockDim.x) adj_tile()[w] = 0u;
@@ -293,28 +296,66 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
           stage ^= 1;
         }
       }
-      for (int base = 0; !STAGE && base < cmax; base += kSlotLanes) {
-        const int k = base + hl;
-        const bool kv = k < cnt;
-        const uint32_t e = kv ? e_cur : 0u;
-        // next chunk's entry, requested now (always inside the row: vcap >= 32;
-        // past the slot's count it is read but not used)
-        e_cur = row[k + kSlotLanes < a.vcap ? k + kSlotLanes : k];
-        bool acc;
-        {
-          // lanes past their slot's last entry (e = 0) evaluate a stand-in and
-          // accept nothing: no branch around the pair
-          T sx = T(0), sy = T(0), sz = T(0);
-          if constexpr (MIXED) {
-            const float4 U = unit_shift[e & 31u];
-            const float2 sxy = mul2(f2(U.x, U.y), f2(dcs, dcs));
-            sx = sxy.x;
-            sy = sxy.y;
-            sz = U.z * dcs;
+      if constexpr (!MIXED) {
+        // FP64: first the test of the entries in FP32 (the exact test inside the
+        // rounding band), the accepted ones compacted in order, then their fluxes
+        // with every lane at work.  Run under the test's branch, the flux (60
+        // instructions of the FP64 pipe, which bounds it) took as many passes
+        // over the slot as it has entries: 65k ejecta, 2 steps, 2.45 -> 1.69 ms.
+        const int ex = exponent_of(g.dc);
+        const float dct = f32_scaled(g.dc, ex), band64 = 0x1p-12f * dct * dct;
+        const float khdi32 = a.kh_f * f32_scaled(Ai.w, ex);
+        for (int seg = 0; seg < cmax; seg += kPassCap) {
+          const int seg_end = min(cmax, seg + kPassCap);
+          int kept = 0;                                 // accepted of this segment (the same in the slot's lanes)
+          for (int base = seg; base < seg_end; base += kSlotLanes) {
+            const int k = base + hl;
+            const bool kv = k < cnt;
+            const uint32_t e = kv ? e_cur : 0u;
+            e_cur = row[k + kSlotLanes < a.vcap ? k + kSlotLanes : k];
+            const uint32_t j = e >> 5;
+            const V4 Aj = A[j];
+            const float tx = f32_scaled(Aj.x - Ai.x, ex);
+            const float ty = DIM >= 2 ? f32_scaled(Aj.y - Ai.y, ex) : 0.f;
+            const float tz = DIM >= 3 ? f32_scaled(Aj.z - Ai.z, ex) : 0.f;
+            const float R = fmaf(a.kh_f, f32_scaled(Aj.w, ex), khdi32);
+            const float diff = fmaf(-R, R, Pair<true, DIM>::r2_of(tx, ty, tz));
+            bool acc = kv && diff < 0.f;
+            if (kv && fabsf(diff) <= band64) acc = exact_accept(a, DIM, a.perm[ii], a.perm[j]);
+            const unsigned mine = (__ballot_sync(0xffffffffu, acc) >> (half * kSlotLanes)) & ((1u << kSlotLanes) - 1u);
+            if (acc) passed[warp][half][kept + __popc(mine & ((1u << hl) - 1u))] = j;
+            kept += __popc(mine);
           }
-          acc = fw.pair_listed(a, ii, Ai, Bi, Ci, ui, (int64_t)(e >> 5), sx, sy, sz, khdi, band, te, kv);
+          nacc += hl == 0 ? (unsigned)kept : 0u;
+          __syncwarp();
+          for (int k = hl; k < kept; k += kSlotLanes) fw.pair(a, ii, Ai, Bi, Ci, ui, passed[warp][half][k], T(0), T(0), T(0));
+          __syncwarp();                                 // `passed` is rewritten by the next segment or slot
         }
-        nacc += acc ? 1u : 0u;                        // this lane's accepted entries
+      }
+      if constexpr (MIXED && !STAGE) {
+        for (int base = 0; base < cmax; base += kSlotLanes) {
+          const int k = base + hl;
+          const bool kv = k < cnt;
+          const uint32_t e = kv ? e_cur : 0u;
+          // next chunk's entry, requested now (always inside the row: vcap >= 32;
+          // past the slot's count it is read but not used)
+          e_cur = row[k + kSlotLanes < a.vcap ? k + kSlotLanes : k];
+          bool acc;
+          {
+            // lanes past their slot's last entry (e = 0) evaluate a stand-in and
+            // accept nothing: no branch around the pair
+            T sx = T(0), sy = T(0), sz = T(0);
+            if constexpr (MIXED) {
+              const float4 U = unit_shift[e & 31u];
+              const float2 sxy = mul2(f2(U.x, U.y), f2(dcs, dcs));
+              sx = sxy.x;
+              sy = sxy.y;
+              sz = U.z * dcs;
+            }
+            acc = fw.pair_listed(a, ii, Ai, Bi, Ci, ui, (int64_t)(e >> 5), sx, sy, sz, khdi, band, te, kv);
+          }
+          nacc += acc ? 1u : 0u;                        // this lane's accepted entries
+        }
       }
       fw.fold();
 #pragma unroll

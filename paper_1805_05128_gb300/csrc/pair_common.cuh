@@ -553,13 +553,13 @@ struct FwdAcc {
     }
   }
 
-  // A listed candidate j of slot i (never i itself): the interaction test of
-  // the scan, then the flux of an interacting pair.  Mixed: FP32 test on the
-  // flux's own separation, decided in FP64 (oracle order) within the band
-  // |r^2 - (kappa h_ij)^2| <= band, where FP32 rounding could flip it; FP64:
-  // the oracle's test.  Returns whether the pair interacts.
+  // A listed candidate j of slot i (never i itself) in mixed precision: the
+  // interaction test of the scan, then the flux of an interacting pair.  FP32
+  // test on the flux's own separation, decided in FP64 (oracle order) within the
+  // band |r^2 - (kappa h_ij)^2| <= band, where FP32 rounding could flip it.
+  // Returns whether the pair interacts.
   __device__ __forceinline__ bool pair_listed(const PairArgs& a, int64_t i, const V4& Ai, const V4& Bi,
-                                              const VC& Ci, int ui, int64_t j, T sx, T sy, T sz, T khdi,
+                                              const VC& Ci, int ui, uint32_t j, T sx, T sy, T sz, T khdi,
                                               float band, unsigned& nexact, bool valid = true) {
     const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
     const V4* __restrict__ B = reinterpret_cast<const V4*>(a.B);
@@ -583,36 +583,24 @@ struct FwdAcc {
     T dx, dy, dz;
     separation(Ai, Aj, sx, sy, sz, dx, dy, dz);
     const T r2 = P::r2_of(dx, dy, dz);
-    bool acc;
-    if (MIXED) {
-      const T R = fmaf((T)a.kh_f, Aj.w, khdi);
-      const T diff = fmaf(-R, R, r2);
-      acc = valid && diff < T(0);
-      if (valid && fabsf(diff) <= band) {
-        ++nexact;
-        acc = exact_accept(a, DIM, a.perm[i], a.perm[j]);
-      }
-    } else {
-      T ex, ey, ez;
-      P::sep(true, Ai, Aj, T(0), T(0), T(0), ex, ey, ez);   // x_j - x_i, oracle order
-      const double R = __dmul_rn(a.kh, __dadd_rn(Ai.w, Aj.w));
-      acc = valid && P::r2_of(ex, ey, ez) < __dmul_rn(R, R);
+    const T R = fmaf((T)a.kh_f, Aj.w, khdi);
+    const T diff = fmaf(-R, R, r2);
+    bool acc = valid && diff < T(0);
+    if (valid && fabsf(diff) <= band) {
+      ++nexact;
+      acc = exact_accept(a, DIM, a.perm[i], a.perm[j]);
     }
-    if constexpr (kX2) {
-      // Branch-free: every listed entry runs the flux arithmetic, and the
-      // kernel derivative is set to zero where the pair does not interact
-      // (such entries lie at q >= kappa, where W' vanishes anyway; the select
-      // keeps the exact pair set).  With ~86 % of the entries interacting the
-      // lanes would run the flux almost always; the branches and their
-      // reconvergence cost more than the idle arithmetic.  The side outputs
-      // (rare: a unit boundary, a pair query) keep their branch.
-      flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2, acc && r2 > T(0));
-      if constexpr (EXTRA) {
-        if (acc) dmax = Aj.w > dmax ? Aj.w : dmax;
-        if (acc && r2 > T(0)) side_outputs(a, i, ui, j);
-      }
-    } else {
-      if (acc) flux_at(a, i, Ai, Bi, Ci, ui, j, Aj, Bj, Cj, dx, dy, dz, r2);
+    // Branch-free: every listed entry runs the flux arithmetic, and the
+    // kernel derivative is set to zero where the pair does not interact
+    // (such entries lie at q >= kappa, where W' vanishes anyway; the select
+    // keeps the exact pair set).  With ~86 % of the entries interacting the
+    // lanes would run the flux almost always; the branches and their
+    // reconvergence cost more than the idle arithmetic.  The side outputs
+    // (rare: a unit boundary, a pair query) keep their branch.
+    flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2, acc && r2 > T(0));
+    if constexpr (EXTRA) {
+      if (acc) dmax = Aj.w > dmax ? Aj.w : dmax;
+      if (acc && r2 > T(0)) side_outputs(a, i, ui, j);
     }
     return acc;
   }

@@ -114,3 +114,37 @@ def test_instances_share_groups(precision):
                 assert np.allclose(g[k][lo:hi], o[k], rtol=0, atol=1e-5 * np.max(np.abs(o[k]))), (b, k)
         one.close()
     sim.close()
+
+
+def _check_step(prob, beta):
+    """One FP64 step with lists against the oracle's."""
+    from paper_1805_05128_gb300 import Simulation
+    sim = Simulation(prob, precision="fp64", units=0, cell_beta=beta)
+    sim.step(2)
+    g = sim.numpy()
+    assert sim.read_status() == 0
+    half = sim.pair_counts()[0]
+    p, s = O.from_problem(prob)
+    O.step(p, s, 2)
+    for k in ("x", "vx", "rho", "E", "ax", "drho", "dE"):
+        ref = getattr(s, k)
+        assert np.max(np.abs(g[k] - ref)) <= 1e-10 * np.max(np.abs(ref)), k
+    _, sd = O.from_problem(prob)
+    for k in "xyz"[: prob.dim]:
+        getattr(sd, k)[:] = g[k]
+    sd.d[:] = g["d"]
+    assert half == len(O.pairs(p, sd, "cells")[0])
+    sim.close()
+
+
+@pytest.mark.parametrize("beta", [0.01, 0.15, 0.4])
+def test_fp64_lists_longer_than_one_segment(beta):
+    """Lists of up to several hundred entries (256 to a segment of the evaluation), most of them rejected at beta = 0.4."""
+    prob = _gas(_lattice((11, 10, 9)))
+    prob.eta = 2.15
+    _check_step(prob, beta)
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -90, 2.0 ** 90])
+def test_fp64_lists_in_any_length_unit(scale):
+    _check_step(_gas(_lattice((7, 6, 5)) * scale, sizes=scale), 0.15)
