@@ -39,7 +39,7 @@
 // order as the oracle, so the pair set is the FP64 one.  (FP64 handles tested
 // every candidate in FP64 before, 12 instructions of a pipe 64 times narrower
 // than FP32's: a third of their pair kernel.)  Mixed per-particle sums are
-// Kahan-compensated; each lane adds its pairs in candidate order.
+// Kahan-compensated; each slot adds its pairs in candidate order.
 #include "pair_common.cuh"
 
 namespace csph {
@@ -51,7 +51,7 @@ constexpr int kRowCap = 112;   // list entries per slot between flushes (row str
 constexpr int kSegs = 2;       // segments per scan before a flush
 constexpr int kSpan = 16;      // cells a segment may span along x (bounds the FP32 frame)
 
-template <bool MIXED, int DIM, int MODE, bool HLL = false, bool EXTRA = true>
+template <bool MIXED, int DIM, int MODE, int G, bool HLL = false, bool EXTRA = true>
 __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kModeFwd2) ? (MIXED ? 4 : 3)
                                                  : (MODE == kModeGrad ? (MIXED ? 5 : 3) : (MIXED ? 6 : 4)))
     k_pair(PairArgs a) {
@@ -64,13 +64,17 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
   using V4 = typename P::V4;
   using V2 = typename P::V2;
   using VC = typename P::VC;
-  __shared__ uint16_t list[kWarps][32][kRowCap + 2];         // [warp][lane][entry]: cell code << 11 | offset
+  constexpr int kHomes = 32 / G;                              // slots per group
+  constexpr int kCap = G == 1 ? kRowCap : 2 * kRowCap;
+  constexpr bool kOrdered = MIXED && G > 1;                   // the sums take the pairs in candidate order
+  __shared__ uint16_t list[kWarps][kHomes][kCap + 2];        // [warp][slot][entry]: cell code << 11 | offset
   __shared__ float4 cand[kWarps][32];                        // candidates that survived the cull: x, y, z, d (FP32)
   __shared__ int2 cand_ent[kWarps][32];                      // their entry in the segment's frame, their slot
   __shared__ float4 nb_tab[kWarps][kSegs][27];               // per segment and cell code: first slot (bits), shift x, y, z
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
+  const int home = lane / G, hl = lane % G;                   // the lane's slot in the group, its place in the slot
   const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
   const V4* __restrict__ B = reinterpret_cast<const V4*>(a.B);
   const VC* __restrict__ C = reinterpret_cast<const VC*>(a.C);
@@ -82,8 +86,8 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
   for (; (int64_t)(q * (unsigned)a.group) < a.n;) {
     const int h0 = (int)(q * (unsigned)a.group);
     const long long t_start = a.load_timed ? clock64() : 0;   // timed unit loads
-    const int i = h0 + lane;
-    const bool act = lane < a.group && i < a.n;
+    const int i = h0 + home;
+    const bool act = home < a.group && i < a.n;
     const int ii = act ? i : h0;
     int b = 0;
     if (a.n_inst > 1) {  // instance of this slot: binary search of the slot offsets
@@ -124,12 +128,13 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       if (DIM >= 2) fw.gVi[1] = GV[a.n + ii];
       if (DIM >= 3) fw.gVi[2] = GV[2 * a.n + ii];
     }
-    auto pair_flux = [&](int64_t j, T sx, T sy, T sz) { fw.pair(a, i, Ai, Bi, Ci, ui, j, sx, sy, sz); };
 
     // SPH gradients (GRAD): grad q_i = sum_j V_j (q_j - q_i) (-W'_ij) e^R for q = P, v_x, v_y, v_z
     T gP[3] = {T(0), T(0), T(0)}, gV[3][3] = {{T(0), T(0), T(0)}, {T(0), T(0), T(0)}, {T(0), T(0), T(0)}};
-    auto pair_grad = [&](int64_t j, T sx, T sy, T sz) {
-      if (j == i) return;
+    struct GradTerms { bool live; T fP, fv[3], e[3]; };
+    auto grad_terms = [&](int64_t j, T sx, T sy, T sz) -> GradTerms {
+      GradTerms q{};
+      if (j == i) return q;
       const V4 Aj = A[j];
       const V4 Bj = B[j];
       const VC Cj = C[j];
@@ -144,7 +149,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         dz = DIM >= 3 ? __dsub_rn(Aj.z, Ai.z) : 0.0;
       }
       const T r2 = MIXED ? P::r2_of(dx, dy, dz) : fw.r2_fused(dx, dy, dz);
-      if (!positive(r2)) return;
+      if (!positive(r2)) return q;
       T ir, r;
       rsqrt_sqrt(r2, ir, r);
       const T e[3] = {dx * ir, dy * ir, dz * ir};
@@ -163,11 +168,18 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         dv[1] = Bj.y - Bi.y;
         dv[2] = Bj.z - Bi.z;
       }
+      q.live = true;
+      q.fP = f * dP;
+#pragma unroll
+      for (int b = 0; b < 3; ++b) { q.fv[b] = f * dv[b]; q.e[b] = e[b]; }
+      return q;
+    };
+    auto add_grad = [&](const GradTerms& q) {
 #pragma unroll
       for (int b = 0; b < DIM; ++b) {
-        gP[b] += f * dP * e[b];
+        gP[b] = fma_(q.fP, q.e[b], gP[b]);
 #pragma unroll
-        for (int c = 0; c < DIM; ++c) gV[c][b] += f * dv[c] * e[b];
+        for (int c = 0; c < DIM; ++c) gV[c][b] = fma_(q.fv[c], q.e[b], gV[c][b]);
       }
     };
 
@@ -332,18 +344,55 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
 
     auto flush = [&]() {
       nfull += (unsigned)cnt;
-      for (int k = 0; k < cnt; ++k) {
-        const unsigned ent = list[warp][lane][k];
-        // (the two minima change nothing on a finite state; on one with infinite
-        // sizes, which is latched, they keep the accesses in bounds)
-        const float4 t = nb_tab[warp][seg_of][min(ent >> 11, 26u)];
-        const int64_t j = min(__float_as_int(t.x) + (int)(ent & 2047u), n_1);
-        if constexpr (VJP) {
-          pair_vjp(j, (T)t.y, (T)t.z, (T)t.w);
-        } else if constexpr (GRAD) {
-          pair_grad(j, (T)t.y, (T)t.z, (T)t.w);
-        } else {
-          pair_flux(j, (T)t.y, (T)t.z, (T)t.w);
+      if constexpr (kOrdered) {
+        // The slot's lanes evaluate consecutive entries; then each of them adds
+        // the terms in candidate order, so the sums are those of one lane going
+        // through the list.
+        const unsigned group = ((1u << G) - 1u) << (home * G);
+        for (int k0 = 0; k0 < cnt; k0 += G) {
+          const int k = k0 + hl;
+          typename FwdAcc<MIXED, DIM, MODE == kModeFwd2, HLL, EXTRA>::Terms q{};
+          GradTerms qg{};
+          if (k < cnt) {
+            const unsigned ent = list[warp][home][k];
+            const float4 t = nb_tab[warp][seg_of][min(ent >> 11, 26u)];
+            const int64_t j = min(__float_as_int(t.x) + (int)(ent & 2047u), n_1);
+            if constexpr (GRAD) qg = grad_terms(j, (T)t.y, (T)t.z, (T)t.w);
+            else q = fw.terms(a, i, Ai, Bi, Ci, ui, j, (T)t.y, (T)t.z, (T)t.w);
+          }
+          const unsigned live = __ballot_sync(group, GRAD ? qg.live : q.live) >> (home * G);
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            if constexpr (GRAD) {
+              GradTerms r;
+              r.fP = __shfl_sync(group, qg.fP, g, G);
+#pragma unroll
+              for (int c = 0; c < DIM; ++c) {
+                r.fv[c] = __shfl_sync(group, qg.fv[c], g, G);
+                r.e[c] = __shfl_sync(group, qg.e[c], g, G);
+              }
+              if ((live >> g) & 1u) add_grad(r);
+            } else {
+              const auto r = fw.from_lane(q, group, g, G);
+              if ((live >> g) & 1u) fw.add(r);
+            }
+          }
+        }
+      } else {
+        for (int k = hl; k < cnt; k += G) {
+          const unsigned ent = list[warp][home][k];
+          // (the two minima change nothing on a finite state; on one with infinite
+          // sizes, which is latched, they keep the accesses in bounds)
+          const float4 t = nb_tab[warp][seg_of][min(ent >> 11, 26u)];
+          const int64_t j = min(__float_as_int(t.x) + (int)(ent & 2047u), n_1);
+          if constexpr (VJP) {
+            pair_vjp(j, (T)t.y, (T)t.z, (T)t.w);
+          } else if constexpr (GRAD) {
+            const GradTerms q = grad_terms(j, (T)t.y, (T)t.z, (T)t.w);
+            if (q.live) add_grad(q);
+          } else {
+            fw.pair(a, i, Ai, Bi, Ci, ui, j, (T)t.y, (T)t.z, (T)t.w);
+          }
         }
       }
       cnt = 0;
@@ -457,7 +506,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         const int r0 = __shfl_sync(0xffffffffu, rs0, r), r1 = __shfl_sync(0xffffffffu, rs1, r);
         const int oy = DIM >= 2 ? r % 3 - 1 : 0, oz = DIM >= 3 ? r / 3 - 1 : 0;
         const int rc = 3 * (oy + 1) + 9 * (oz + 1);            // code of the row's ox = -1 cell
-        if (mine) ncand += (unsigned)(a.cell_start[rb + (cx + 1 < nx ? cx + 2 : nx)] - a.cell_start[rb + (cx > 0 ? cx - 1 : 0)]);
+        if (mine && hl == 0) ncand += (unsigned)(a.cell_start[rb + (cx + 1 < nx ? cx + 2 : nx)] - a.cell_start[rb + (cx > 0 ? cx - 1 : 0)]);
         for (int base = r0; base < r1; base += 32) {
           const int j = base + lane;
           const bool jv = j < r1;
@@ -480,32 +529,55 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
             cand_ent[warp][c] = make_int2(((rc + 1 + relx) << 11) | (off & 2047), j);
           }
           // a chunk adds at most nc entries to a list: flush first if one could overflow
-          if (__any_sync(0xffffffffu, cnt > kRowCap - nc)) flush();
+          if (__any_sync(0xffffffffu, cnt > kCap - nc)) flush();
           __syncwarp();
           const int mybase = cx_seg << 11;
 #pragma unroll 4
-          for (int c = 0; c < nc; ++c) {
+          for (int c0 = 0; c0 < nc; c0 += G) {
+            const int c = c0 + hl;                            // G > 1: the slot's lanes test consecutive candidates
             const float4 Sc = cand[warp][c];
             const float r2 = Pair<true, DIM>::r2_of(Sc.x - H.x, DIM >= 2 ? Sc.y - H.y : 0.f, DIM >= 3 ? Sc.z - H.z : 0.f);
             const float R = fmaf(a.kh_f, Sc.w, H.w);
             const float diff = fmaf(-R, R, r2);              // r^2 - R^2
-            bool acc = diff < 0.f;
-            if (fabsf(diff) <= band) {                        // too close to call in FP32: FP64 decides
+            const bool cv = G == 1 || c < nc;                // (past nc: an old candidate, not used)
+            bool acc = cv && diff < 0.f;
+            if (cv && fabsf(diff) <= band) {                  // too close to call in FP32: FP64 decides
               const int jc = cand_ent[warp][c].y;
               ++nexact;
               acc = jc == i || exact_accept(a, DIM, a.perm[i], a.perm[jc]);
             }
-            if (acc) list[warp][lane][cnt++] = (uint16_t)(cand_ent[warp][c].x - mybase);
+            if constexpr (G == 1) {
+              if (acc) list[warp][home][cnt++] = (uint16_t)(cand_ent[warp][c].x - mybase);
+            } else {
+              const unsigned took = (__ballot_sync(0xffffffffu, acc) >> (home * G)) & ((1u << G) - 1u);
+              if (acc) list[warp][home][cnt + __popc(took & ((1u << hl) - 1u))] = (uint16_t)(cand_ent[warp][c].x - mybase);
+              cnt += __popc(took);
+            }
           }
           __syncwarp();   // the candidate buffer is rewritten by the next chunk
         }
       }
       ++seg;
     }
+    __syncwarp();
     flush();
+    // unordered sums: the slot's lanes hold a part each
+    [[maybe_unused]] auto lanes_sum = [](T& v) {
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    };
+    const bool owner = act && hl == 0;
 
     if constexpr (GRAD) {
-      if (act) {
+      if constexpr (G > 1 && !kOrdered) {
+#pragma unroll
+        for (int b1 = 0; b1 < 3; ++b1) {
+          lanes_sum(gP[b1]);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) lanes_sum(gV[c][b1]);
+        }
+      }
+      if (owner) {
         V4* GP = reinterpret_cast<V4*>(a.gP);
         V4* GV = reinterpret_cast<V4*>(a.gV);
         const T rs = (T)a.rscale;                      // undo the volume and W' scales (powers of two)
@@ -520,7 +592,12 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         }
       }
     } else if constexpr (VJP) {
-      if (act) {
+      if constexpr (G > 1) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) { lanes_sum(s_bx[k].s); lanes_sum(s_bv[k].s); }
+        lanes_sum(s_bP.s); lanes_sum(s_bZ.s); lanes_sum(s_bV.s); lanes_sum(s_bd.s); lanes_sum(s_brho.s);
+      }
+      if (owner) {
         double* o = a.vjp_out + 11 * (int64_t)a.perm[i];
 #pragma unroll
         for (int k = 0; k < 3; ++k) { o[k] = (double)s_bx[k].s; o[3 + k] = (double)s_bv[k].s; }
@@ -531,12 +608,24 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
         o[10] = MIXED ? (double)s_brho.s : -2.0 * (double)Ri.x * (double)s_brho.s;
       }
     } else {
-      if (act) {
+      fw.fold();
+      if constexpr (G > 1) {
+        if constexpr (!kOrdered) {
+          lanes_sum(fw.s_rho.s); lanes_sum(fw.s_fx.s); lanes_sum(fw.s_fy.s); lanes_sum(fw.s_fz.s); lanes_sum(fw.s_q.s);
+        }
+        if constexpr (EXTRA) {
+#pragma unroll
+          for (int o = G / 2; o > 0; o >>= 1) {
+            const T other = __shfl_xor_sync(0xffffffffu, fw.dmax, o);
+            fw.dmax = other > fw.dmax ? other : fw.dmax;
+          }
+        }
+      }
+      if (owner) {
         nfull -= 1;   // the self pair
-        fw.fold();
         fw.write(a, i, nfull);
       }
-      warp_counters(a, act, nfull, ncand, MIXED ? nexact : 0u, ui, lane,
+      warp_counters(a, owner, nfull, ncand, MIXED ? nexact : 0u, ui, lane,
                     a.load_timed ? (unsigned)(clock64() - t_start) : 0u);
     }
     __syncwarp();     // the segment tables and lists are rewritten by the next group
@@ -547,21 +636,20 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
 
 // Persistent grid: SMs x resident CTAs per SM, capped by the handle's
 // pair_blocks_per_sm (0 = as many as fit) and by the number of groups.
-// Groups hold 32 slots; a system too small to give every SM four warps takes
-// 16 or 8 slots per group, so that more SMs share its scan.
-template <bool MIXED, int DIM, int MODE, bool HLL, bool EXTRA = true>
-cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
+template <bool MIXED, int DIM, int MODE, int G, bool HLL, bool EXTRA>
+cudaError_t launch_lanes(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
   static int sms = 0, per_sm = 0;
   if (sms == 0) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<MIXED, DIM, MODE, HLL, EXTRA>, kPairBlock, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<MIXED, DIM, MODE, G, HLL, EXTRA>, kPairBlock, 0);
     if (per_sm < 1) per_sm = 1;
   }
   PairArgs a = args;
-  a.group = 32;
-  while (a.group > 8 && a.n < (int64_t)4 * sms * a.group) a.group >>= 1;
+  a.group = 32 / G;
+  // a group of fewer slots while not every SM has four warps at work
+  while (a.group > (G == 1 ? 8 : 2) && a.n < (int64_t)4 * sms * a.group) a.group >>= 1;
   const int64_t groups = (a.n + a.group - 1) / a.group;
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
   // few groups: one CTA per SM until each holds a group per warp (a CTA's warps
@@ -572,8 +660,31 @@ cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st)
   // resident while that one still runs are packed onto the SMs with room left
   // instead of being spread over all of them (6k particles in a plane, FP64, a
   // step: 0.30 ms spread, 0.38 ms packed).
-  k_pair<MIXED, DIM, MODE, HLL, EXTRA><<<grid, kPairBlock, 0, st>>>(a);
+  k_pair<MIXED, DIM, MODE, G, HLL, EXTRA><<<grid, kPairBlock, 0, st>>>(a);
   return cudaGetLastError();
+}
+
+// Lanes per slot.  One lane per slot does the least work per pair, but a group
+// of 32 slots is then one chain of ~600 candidate tests and ~80 fluxes: 147 us
+// for 32k particles, whose groups do not fill the chip once.  With four lanes a
+// slot's candidates and fluxes are shared out: mixed, pair kernel, 1.5k
+// particles 70 -> 41 us, 32k 147 -> 104, 58k 165 -> 141, but 77k 165 -> 185
+// (in a plane 24k 40 -> 31, 43k 41 -> 48), with the sums still taken in
+// candidate order, the same bits.  FP64 handles, whose fluxes fill the FP64
+// pipe from either form, take four lanes at any size, so that their sums'
+// rounding does not depend on how many particles share the handle: 1.5k
+// 219 -> 101 us, 32k 572 -> 370, 203k 2175 -> 2095; a 97k plane 261 -> 281.
+template <bool MIXED, int DIM, int MODE, bool HLL, bool EXTRA = true>
+cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
+  if constexpr (!MIXED) {
+    return launch_lanes<MIXED, DIM, MODE, 4, HLL, EXTRA>(args, blocks_per_sm, st);
+  } else {
+    if constexpr (MODE != kModeVjp) {
+      constexpr int64_t few = DIM == 3 ? 65536 : 32768;
+      if (args.n <= few) return launch_lanes<MIXED, DIM, MODE, 4, HLL, EXTRA>(args, blocks_per_sm, st);
+    }
+    return launch_lanes<MIXED, DIM, MODE, 1, HLL, EXTRA>(args, blocks_per_sm, st);
+  }
 }
 
 template <bool MIXED, int MODE, bool HLL, bool EXTRA>

@@ -511,18 +511,63 @@ struct FwdAcc {
     return s;
   }
 
+  // One pair's contribution to the sums: u w (continuity, the product unrounded
+  // in the sum), the momentum flux F e and the energy flux.  live = false: none.
+  struct Terms {
+    bool live;
+    T u, w, F, fx, fy, fz, q, ex, ey, ez, qv;
+  };
+
+  __device__ __forceinline__ void add(const Terms& t) {
+    s_rho.add_product(t.u, t.w);
+    if constexpr (kX2) {
+      k_fxy.add(f2(t.fx, t.fy));
+      k_fzq.add(f2(t.fz, t.q));
+    } else if constexpr (MIXED) {
+      s_fx.add(t.fx);
+      if (DIM >= 2) s_fy.add(t.fy);
+      if (DIM >= 3) s_fz.add(t.fz);
+      s_q.add(t.q);
+    } else {
+      s_fx.add_product(t.F, t.ex);
+      if (DIM >= 2) s_fy.add_product(t.F, t.ey);
+      if (DIM >= 3) s_fz.add_product(t.F, t.ez);
+      s_q.add_product(t.F, t.qv);
+    }
+  }
+
+  // The terms that lane g of the slot's `width` lanes holds (mixed precision).
+  static __device__ __forceinline__ Terms from_lane(const Terms& t, unsigned mask, int g, int width) {
+    Terms r = t;
+    r.u = __shfl_sync(mask, t.u, g, width);
+    r.w = __shfl_sync(mask, t.w, g, width);
+    r.fx = __shfl_sync(mask, t.fx, g, width);
+    r.fy = __shfl_sync(mask, t.fy, g, width);
+    r.fz = __shfl_sync(mask, t.fz, g, width);
+    r.q = __shfl_sync(mask, t.q, g, width);
+    return r;
+  }
+
   __device__ __forceinline__ void pair(const PairArgs& a, int64_t i, const V4& Ai, const V4& Bi, const VC& Ci,
                                        int ui, int64_t j, T sx, T sy, T sz) {
+    terms<true>(a, i, Ai, Bi, Ci, ui, j, sx, sy, sz);
+  }
+
+  // The pair's terms; ADD: added to the sums here (each form by its own branch,
+  // which keeps the terms of the other out of the registers).
+  template <bool ADD = false>
+  __device__ __forceinline__ Terms terms(const PairArgs& a, int64_t i, const V4& Ai, const V4& Bi, const VC& Ci,
+                                         int ui, int64_t j, T sx, T sy, T sz) {
     const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
     const V4* __restrict__ B = reinterpret_cast<const V4*>(a.B);
     const VC* __restrict__ C = reinterpret_cast<const VC*>(a.C);
-    if (j == i) return;       // the scan keeps the self pair (r = 0); it has no flux
+    if (j == i) return Terms{};   // the scan keeps the self pair (r = 0); it has no flux
     const V4 Aj = A[j];
     const V4 Bj = B[j];
     const VC Cj = C[j];
     T dx, dy, dz;
     separation(Ai, Aj, sx, sy, sz, dx, dy, dz);
-    flux_at(a, i, Ai, Bi, Ci, ui, j, Aj, Bj, Cj, dx, dy, dz, MIXED ? P::r2_of(dx, dy, dz) : r2_fused(dx, dy, dz));
+    return flux_at<ADD>(a, i, Ai, Bi, Ci, ui, j, Aj, Bj, Cj, dx, dy, dz, MIXED ? P::r2_of(dx, dy, dz) : r2_fused(dx, dy, dz));
   }
 
   // r^2 of the flux arithmetic (the interaction test has its own operation order)
@@ -597,7 +642,7 @@ struct FwdAcc {
     // lanes would run the flux almost always; the branches and their
     // reconvergence cost more than the idle arithmetic.  The side outputs
     // (rare: a unit boundary, a pair query) keep their branch.
-    flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2, acc && r2 > T(0));
+    add(flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2, acc && r2 > T(0)));
     if constexpr (EXTRA) {
       if (acc) dmax = Aj.w > dmax ? Aj.w : dmax;
       if (acc && r2 > T(0)) side_outputs(a, i, ui, j);
@@ -611,9 +656,9 @@ struct FwdAcc {
   // side, P* and W' are the same bits).
   // live = false: the terms are computed with W' = 0 (and a positive stand-in
   // for r^2 = 0), so they add zeros; the caller then needs no branch.
-  __device__ __forceinline__ void flux_x2(const PairArgs& a, const float4& Ai, const float4& Bi,
+  __device__ __forceinline__ Terms flux_x2(const PairArgs& a, const float4& Ai, const float4& Bi,
                                           const float4& Ci, const float4& Aj, const float4& Bj, const float4& Cj,
-                                          float dx, float dy, float dz, float r2, bool live = true) {
+                                          float dx, float dy, float dz, float r2, bool live = true) const {
     if (!(r2 > 0.f)) r2 = 1.f;                       // coincident particles: no direction (live is false)
     const float ir = rsqrtf(r2);
     const float r = r2 * ir;
@@ -638,7 +683,7 @@ struct FwdAcc {
     const float hij = a.eta_half_f * add_(Ai.w, Aj.w);
     float dW = dw_fast<float, DIM, KERN>(a.kernel, a.kappa_f, r, hij, a.wscale_f);
     dW = live ? dW : 0.f;
-    add_x2(Bj.w * (-du), dW, mul_(mul_(mul_(Bi.w, Bj.w), Ps), dW), exy, ez, du);
+    return terms_x2(Bj.w * (-du), dW, mul_(mul_(mul_(Bi.w, Bj.w), Ps), dW), exy, ez, du);
   }
 
   // flux_x2 for a pair that interacts and whose r^2 and Z_i + Z_j are normal
@@ -647,9 +692,9 @@ struct FwdAcc {
   // cell search takes it (387k plate: 2.12 -> 2.01 ms per 3 steps); in the list
   // kernel, which the L1 data pipe bounds (88 % of its wavefronts), 7 % fewer
   // instructions this way changed nothing, and its entries need the selects.
-  __device__ __forceinline__ void regular_flux_x2(const PairArgs& a, const float4& Ai, const float4& Bi, const float4& Ci,
+  __device__ __forceinline__ Terms regular_flux_x2(const PairArgs& a, const float4& Ai, const float4& Bi, const float4& Ci,
                                                   const float4& Aj, const float4& Bj, const float4& Cj, float dx, float dy,
-                                                  float dz, float r2) {
+                                                  float dz, float r2) const {
     const float ir = rsqrt_ftz(r2);
     const float r = r2 * ir;
     const float2 exy = mul2(f2(dx, dy), f2(ir, ir));
@@ -664,15 +709,21 @@ struct FwdAcc {
     const float Ps = mul_(numP, izs), du = mul_(numu, izs);   // P*; v* - v_i^R
     const float hij = a.eta_half_f * add_(Ai.w, Aj.w);
     const float dW = dw_fast<float, DIM, KERN, true>(a.kernel, a.kappa_f, r, hij, a.wscale_f);
-    add_x2(Bj.w * (-du), dW, mul_(mul_(mul_(Bi.w, Bj.w), Ps), dW), exy, ez, du);
+    return terms_x2(Bj.w * (-du), dW, mul_(mul_(mul_(Bi.w, Bj.w), Ps), dW), exy, ez, du);
   }
 
-  // continuity term u (-W'), momentum F e (without its factor 2, carried by
-  // fscale; exact), energy F (v* - v_i^R)
-  __device__ __forceinline__ void add_x2(float u, float dW, float F, float2 exy, float ez, float du) {
-    s_rho.add_product(u, -dW);
-    k_fxy.add(mul2(f2(F, F), exy));
-    k_fzq.add(f2(mul_(F, ez), mul_(F, du)));
+  // momentum F e without its factor 2 (carried by fscale; exact), energy F (v* - v_i^R)
+  static __device__ __forceinline__ Terms terms_x2(float u, float dW, float F, float2 exy, float ez, float du) {
+    Terms t{};
+    const float2 f = mul2(f2(F, F), exy);
+    t.live = true;
+    t.u = u;
+    t.w = -dW;
+    t.fx = f.x;
+    t.fy = f.y;
+    t.fz = mul_(F, ez);
+    t.q = mul_(F, du);
+    return t;
   }
 
   static __device__ __forceinline__ bool regular_x2(float r2, const float4& Ci, const float4& Cj) {
@@ -692,16 +743,23 @@ struct FwdAcc {
     return gR;
   }
 
-  __device__ __forceinline__ void flux_at(const PairArgs& a, int64_t i, const V4& Ai, const V4& Bi, const VC& Ci,
+  template <bool ADD>
+  __device__ __forceinline__ Terms flux_at(const PairArgs& a, int64_t i, const V4& Ai, const V4& Bi, const VC& Ci,
                                           int ui, int64_t j, const V4& Aj, const V4& Bj, const VC& Cj, T dx, T dy,
                                           T dz, T r2) {
     if constexpr (EXTRA) dmax = Aj.w > dmax ? Aj.w : dmax;
-    if (!positive(r2)) return;  // coincident particles: no direction, no flux
+    if (!positive(r2)) return Terms{};  // coincident particles: no direction, no flux
     if constexpr (kX2) {
-      if (regular_x2(r2, Ci, Cj)) regular_flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2);
-      else flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2);
+      Terms t{};
+      if (regular_x2(r2, Ci, Cj)) {
+        t = regular_flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2);
+        if constexpr (ADD) add(t);
+      } else {
+        t = flux_x2(a, Ai, Bi, Ci, Aj, Bj, Cj, dx, dy, dz, r2);
+        if constexpr (ADD) add(t);
+      }
       side_outputs(a, i, ui, j);
-      return;
+      return t;
     }
     T ir, r;
     rsqrt_sqrt(r2, ir, r);
@@ -793,20 +851,25 @@ struct FwdAcc {
     }
     // momentum flux along e, without its factor 2 (carried by fscale; exact)
     const T F = mul_(mul_(mul_(Bi.w, Bj.w), Ps), dW);
+    Terms t{};
+    t.live = true;
+    t.u = Bj.w * cr;
+    t.w = -dW;
     if constexpr (MIXED) {
-      s_rho.add(Bj.w * cr * (-dW));
-      s_fx.add(mul_(F, ex));
-      if (DIM >= 2) s_fy.add(mul_(F, ey));
-      if (DIM >= 3) s_fz.add(mul_(F, ez));
-      s_q.add(mul_(F, qv));
+      t.fx = mul_(F, ex);
+      t.fy = mul_(F, ey);
+      t.fz = mul_(F, ez);
+      t.q = mul_(F, qv);
     } else {
-      s_rho.add_product(Bj.w * cr, -dW);
-      s_fx.add_product(F, ex);
-      if (DIM >= 2) s_fy.add_product(F, ey);
-      if (DIM >= 3) s_fz.add_product(F, ez);
-      s_q.add_product(F, qv);
+      t.F = F;
+      t.ex = ex;
+      t.ey = ey;
+      t.ez = ez;
+      t.qv = qv;
     }
+    if constexpr (ADD) add(t);
     side_outputs(a, i, ui, j);
+    return t;
   }
 
   // EXTRA: the optional pair output and the unit adjacency of an interacting pair.
