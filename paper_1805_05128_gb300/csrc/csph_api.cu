@@ -30,24 +30,66 @@ int cuda_fail(sph_handle* h, const char* what, cudaError_t e) {
     if (e_ != cudaSuccess) return cuda_fail((h), #call, e_);  \
   } while (0)
 
-template <typename T>
-cudaError_t dalloc(T** p, size_t count) {
-  *p = nullptr;
-  if (count == 0) count = 1;
-  return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * count);
-}
+// A handle's workspace in one allocation: the arrays are requested first, then
+// laid out (uploaded ones, zeroed ones, the others) and set up with one copy and
+// one memset.  An allocation, copy or free per array cost a handle 1.0 to 1.5 ms
+// from creation to destruction, a tenth of a short differentiable run.
+class Workspace {
+ public:
+  template <typename T>
+  void raw(T** p, size_t count) { add(p, sizeof(T) * count, 2, nullptr); }
+  template <typename T>
+  void zeroed(T** p, size_t count) { add(p, sizeof(T) * count, 1, nullptr); }
+  template <typename T>
+  void upload(T** p, const std::vector<T>& v) { add(p, sizeof(T) * v.size(), 0, v.data()); }
+
+  // Allocates into *base and sets every requested pointer; the copy and the
+  // memset are enqueued on st.
+  cudaError_t commit(void** base, cudaStream_t st) {
+    size_t end[3], at = 0;
+    for (int kind = 0; kind < 3; ++kind) {
+      for (Item& it : items_)
+        if (it.kind == kind) {
+          it.at = at;
+          at += (it.bytes + 255) / 256 * 256;
+        }
+      end[kind] = at;
+    }
+    *base = nullptr;
+    cudaError_t e = cudaMalloc(base, at > 0 ? at : 256);
+    if (e != cudaSuccess) { *base = nullptr; return e; }
+    char* b = static_cast<char*>(*base);
+    std::vector<char> host(end[0]);
+    for (const Item& it : items_) {
+      *it.ptr = b + it.at;
+      if (it.kind == 0 && !it.data.empty()) std::memcpy(host.data() + it.at, it.data.data(), it.bytes);
+    }
+    if (end[0] > 0 && (e = cudaMemcpyAsync(b, host.data(), end[0], cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
+    if (end[1] > end[0] && (e = cudaMemsetAsync(b + end[0], 0, end[1] - end[0], st)) != cudaSuccess) return e;
+    return cudaSuccess;   // (a copy from pageable memory has left `host` when it returns)
+  }
+
+ private:
+  struct Item {
+    void** ptr;
+    size_t bytes, at;
+    int kind;
+    std::vector<char> data;
+  };
+  std::vector<Item> items_;
+
+  template <typename T>
+  void add(T** p, size_t bytes, int kind, const void* data) {
+    Item it{reinterpret_cast<void**>(p), bytes > 0 ? bytes : 1, 0, kind, {}};
+    if (data) it.data.assign(static_cast<const char*>(data), static_cast<const char*>(data) + bytes);
+    items_.push_back(std::move(it));
+  }
+};
 
 void free_all(sph_handle* h) {
-  void* ptrs[] = {h->blk_inst, h->blk_start, h->blk_end, h->inst_blk, h->inst_off, h->part, h->grid, h->dt,
-                  h->inst_cap, h->total_cells, h->cell_count, h->cell_start, h->scan_sums, h->cell_of, h->rank,
-                  h->perm, h->slot_cell, h->slot_unit, h->packA, h->packB, h->packC, h->rho_slot, h->dmax_nbr,
-                  h->load_acc, h->adj_bits, h->unit_off, h->unit_list, h->unit_work, h->unit_total, h->unit_stats,
-                  h->status, h->counters, h->scratch, h->adj_G,
-                  h->adj_GR, h->adj_pair, h->adj_par, h->adj_W, h->adj_store, h->mat_dev, h->vlist, h->vcnt,
-                  h->vref, h->vflag, h->grad_p, h->grad_v, h->adj64_A, h->adj64_B, h->adj64_C,
-                  h->adj64_rho, h->dt_key, h->e_of_c, h->perm_e, h->unit_eoff, h->packAc, h->unit_q, h->unit_t, h->slot_org, h->vinst};
-  for (void* p : ptrs)
+  for (void* p : h->blocks)
     if (p) cudaFree(p);
+  h->blocks.clear();
 }
 
 int check_state(sph_handle* h, const sph_state* s, int dim) {
@@ -199,9 +241,8 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     if (e_ != cudaSuccess) { cuda_fail(h, #call, e_); return bail(SPH_ERR_CUDA); } \
   } while (0)
 
-  CKI(dalloc(&h->mat_dev, h->mat_h.size()));
-  CKI(cudaMemcpy(h->mat_dev, h->mat_h.data(), sizeof(Mat) * h->mat_h.size(), cudaMemcpyHostToDevice));
-  dp.mat = h->mat_dev;
+  Workspace ws;
+  ws.upload(&h->mat_dev, h->mat_h);
 
   // segmented blocks
   std::vector<int32_t> bi;
@@ -218,22 +259,16 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
   h->inst_blk_h.push_back((int32_t)bi.size());
   h->nblk = (int)bi.size();
   const int64_t n = h->n;
-  CKI(dalloc(&h->blk_inst, h->nblk));
-  CKI(dalloc(&h->blk_start, h->nblk));
-  CKI(dalloc(&h->blk_end, h->nblk));
-  CKI(dalloc(&h->inst_blk, n_instances + 1));
-  CKI(dalloc(&h->inst_off, n_instances + 1));
-  CKI(cudaMemcpy(h->blk_inst, bi.data(), sizeof(int32_t) * bi.size(), cudaMemcpyHostToDevice));
-  CKI(cudaMemcpy(h->blk_start, bs.data(), sizeof(int64_t) * bs.size(), cudaMemcpyHostToDevice));
-  CKI(cudaMemcpy(h->blk_end, be.data(), sizeof(int64_t) * be.size(), cudaMemcpyHostToDevice));
-  CKI(cudaMemcpy(h->inst_blk, h->inst_blk_h.data(), sizeof(int32_t) * (n_instances + 1), cudaMemcpyHostToDevice));
-  CKI(cudaMemcpy(h->inst_off, inst_offsets, sizeof(int64_t) * (n_instances + 1), cudaMemcpyHostToDevice));
+  ws.upload(&h->blk_inst, bi);
+  ws.upload(&h->blk_start, bs);
+  ws.upload(&h->blk_end, be);
+  ws.upload(&h->inst_blk, h->inst_blk_h);
+  ws.upload(&h->inst_off, h->inst_off_h);
 
-  CKI(dalloc(&h->part, h->nblk));
-  CKI(dalloc(&h->grid, n_instances));
-  CKI(dalloc(&h->dt, n_instances));
-  CKI(dalloc(&h->inst_cap, n_instances));
-  CKI(dalloc(&h->total_cells, 1));
+  ws.raw(&h->part, h->nblk);
+  ws.raw(&h->grid, n_instances);
+  ws.raw(&h->dt, n_instances);
+  ws.raw(&h->total_cells, 1);
   std::vector<int64_t> caps(n_instances);
   for (int b = 0; b < n_instances; ++b) {
     int64_t nb = inst_offsets[b + 1] - inst_offsets[b];
@@ -242,43 +277,34 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     caps[b] = n_instances == 1 ? p->cell_cap
                                : 1 + (int64_t)((double)(p->cell_cap - n_instances) * (double)nb / (double)n);
   }
-  CKI(cudaMemcpy(h->inst_cap, caps.data(), sizeof(int64_t) * n_instances, cudaMemcpyHostToDevice));
+  ws.upload(&h->inst_cap, caps);
 
   h->cell_cap = p->cell_cap;
-  CKI(dalloc(&h->cell_count, h->cell_cap));
-  CKI(cudaMemset(h->cell_count, 0, sizeof(int32_t) * h->cell_cap));
-  CKI(dalloc(&h->cell_start, h->cell_cap + 1));
-  CKI(dalloc(&h->scan_sums, h->cell_cap / 1024 + 2));
-  CKI(dalloc(&h->cell_of, n));
-  CKI(dalloc(&h->rank, n));
-  CKI(dalloc(&h->perm, n));
-  CKI(dalloc(&h->slot_cell, n));
-  CKI(dalloc(&h->slot_unit, n));
+  ws.zeroed(&h->cell_count, h->cell_cap);
+  ws.raw(&h->cell_start, h->cell_cap + 1);
+  ws.raw(&h->scan_sums, h->cell_cap / 1024 + 2);
+  ws.raw(&h->cell_of, n);
+  ws.raw(&h->rank, n);
+  ws.raw(&h->perm, n);
+  ws.raw(&h->slot_cell, n);
+  ws.raw(&h->slot_unit, n);
   if (p->precision == SPH_PREC_MIXED) {
-    CKI(dalloc(&h->slot_org, (size_t)3 * n));
-    CKI(cudaMemset(h->slot_org, 0, sizeof(double) * 3 * n));
-    h->dp.slot_org = h->slot_org;
-    CKI(dalloc(reinterpret_cast<float4**>(&h->packA), n));
-    CKI(dalloc(reinterpret_cast<float4**>(&h->packB), n));
-    CKI(dalloc(reinterpret_cast<float4**>(&h->packC), n));
+    ws.zeroed(&h->slot_org, (size_t)3 * n);
+    ws.raw(reinterpret_cast<float4**>(&h->packA), n);
+    ws.raw(reinterpret_cast<float4**>(&h->packB), n);
+    ws.raw(reinterpret_cast<float4**>(&h->packC), n);
   } else {
-    CKI(dalloc(reinterpret_cast<D4**>(&h->packA), n));
-    CKI(dalloc(reinterpret_cast<D4**>(&h->packB), n));
-    CKI(dalloc(reinterpret_cast<D2**>(&h->packC), n));
+    ws.raw(reinterpret_cast<D4**>(&h->packA), n);
+    ws.raw(reinterpret_cast<D4**>(&h->packB), n);
+    ws.raw(reinterpret_cast<D2**>(&h->packC), n);
   }
-  CKI(dalloc(&h->rho_slot, n));
-  CKI(dalloc(&h->dmax_nbr, n));
-  CKI(dalloc(&h->dt_key, (size_t)n_instances));
-  {
-    std::vector<long long> inf((size_t)n_instances, LLONG_MAX);
-    CKI(cudaMemcpy(h->dt_key, inf.data(), sizeof(long long) * inf.size(), cudaMemcpyHostToDevice));
-  }
-  CKI(dalloc(&h->status, 1));
-  CKI(cudaMemset(h->status, 0, sizeof(int)));
-  CKI(dalloc(&h->counters, 8));
-  CKI(cudaMemset(h->counters, 0, 8 * sizeof(unsigned long long)));
+  ws.raw(&h->rho_slot, n);
+  ws.raw(&h->dmax_nbr, n);
+  ws.upload(&h->dt_key, std::vector<long long>((size_t)n_instances, LLONG_MAX));
+  ws.zeroed(&h->counters, 8);
+  ws.zeroed(&h->status, 1);
   h->scratch_bytes = (size_t)n * (18 * 8 + 8 + 4 + 4);
-  CKI(cudaMalloc(&h->scratch, h->scratch_bytes));
+  ws.raw(reinterpret_cast<char**>(&h->scratch), h->scratch_bytes);
 
   h->K = p->n_units;
   h->gdim = p->unit_dim;
@@ -286,19 +312,15 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     int K = h->K;
     int nb = grid_for(n, 1024);
     h->unit_work_total = (int64_t)K * nb;
-    CKI(dalloc(&h->load_acc, K));
-    CKI(cudaMemset(h->load_acc, 0, sizeof(unsigned long long) * K));
-    CKI(dalloc(&h->adj_bits, (size_t)K * ((K + 31) / 32)));
-    CKI(cudaMemset(h->adj_bits, 0, sizeof(uint32_t) * K * ((K + 31) / 32)));
-    CKI(dalloc(&h->unit_off, K + 1));
-    CKI(dalloc(&h->unit_list, n));
-    CKI(dalloc(&h->unit_work, 2 * h->unit_work_total + h->unit_work_total / 1024 + 4));
-    CKI(cudaMemset(h->unit_work, 0, sizeof(int32_t) * (2 * h->unit_work_total + h->unit_work_total / 1024 + 4)));
-    CKI(dalloc(&h->unit_total, 1));
-    CKI(cudaMemcpy(h->unit_total, &h->unit_work_total, sizeof(int64_t), cudaMemcpyHostToDevice));
+    ws.zeroed(&h->load_acc, K);
+    ws.zeroed(&h->adj_bits, (size_t)K * ((K + 31) / 32));
+    ws.raw(&h->unit_off, K + 1);
+    ws.raw(&h->unit_list, n);
+    ws.zeroed(&h->unit_work, 2 * h->unit_work_total + h->unit_work_total / 1024 + 4);
+    ws.upload(&h->unit_total, std::vector<int64_t>(1, h->unit_work_total));
     // 5 statistics + 4 balancing scratch per unit, then the statistics' partial sums
     // (up to 16 blocks per unit, 4 values each)
-    CKI(dalloc(&h->unit_stats, (size_t)K * (9 + 16 * 4)));
+    ws.raw(&h->unit_stats, (size_t)K * (9 + 16 * 4));
   }
 
   // order-2 reconstruction: SPH gradients of P and v in slot order
@@ -307,11 +329,11 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
   h->load_timed = p->load_measure == SPH_LOAD_TIME;
   if (h->order2) {
     if (p->precision == SPH_PREC_MIXED) {
-      CKI(dalloc(reinterpret_cast<float4**>(&h->grad_p), n));
-      CKI(dalloc(reinterpret_cast<float4**>(&h->grad_v), (size_t)3 * n));
+      ws.raw(reinterpret_cast<float4**>(&h->grad_p), n);
+      ws.raw(reinterpret_cast<float4**>(&h->grad_v), (size_t)3 * n);
     } else {
-      CKI(dalloc(reinterpret_cast<D4**>(&h->grad_p), n));
-      CKI(dalloc(reinterpret_cast<D4**>(&h->grad_v), (size_t)3 * n));
+      ws.raw(reinterpret_cast<D4**>(&h->grad_p), n);
+      ws.raw(reinterpret_cast<D4**>(&h->grad_v), (size_t)3 * n);
     }
   }
 
@@ -328,50 +350,47 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     const double vol = p->dim == 1 ? 2.0 * rr : (p->dim == 2 ? pi * rr * rr : 4.0 / 3.0 * pi * rr * rr * rr);
     const double cap = p->list_cap > 0 ? (double)p->list_cap : std::ceil((p->dim == 3 ? 2.0 : 3.0) * vol + 32.0);
     h->vcap = (int)std::min(65536.0, std::ceil(cap / 32.0) * 32.0);
-    CKI(dalloc(&h->vlist, (size_t)h->vcap * n));
-    CKI(dalloc(&h->vcnt, n));
+    ws.raw(&h->vlist, (size_t)h->vcap * n);
+    ws.raw(&h->vcnt, n);
     const size_t ni = (size_t)n_instances;
-    CKI(dalloc(&h->vref, (size_t)4 * n + 10 * ni));
-    CKI(cudaMemset(h->vref, 0, sizeof(double) * (4 * n + 10 * ni)));
+    ws.zeroed(&h->vref, (size_t)4 * n);
     // per instance: U = 0 (also its FP32 copy), one step since the build; empty accumulators
-    h->vframe = h->vref + (size_t)4 * n;
-    h->vacc = reinterpret_cast<VAcc*>(h->vframe + 6 * ni);
     std::vector<double> frame0(6 * ni, 0.0);
     for (size_t b = 0; b < ni; ++b) frame0[6 * b + 3] = 1.0;
-    CKI(cudaMemcpy(h->vframe, frame0.data(), sizeof(double) * frame0.size(), cudaMemcpyHostToDevice));
+    ws.upload(&h->vframe, frame0);
     const VAcc acc0{LLONG_MIN, {INT_MAX, INT_MAX, INT_MAX}, {INT_MIN, INT_MIN, INT_MIN}};
-    std::vector<VAcc> accs(ni, acc0);
-    CKI(cudaMemcpy(h->vacc, accs.data(), sizeof(VAcc) * ni, cudaMemcpyHostToDevice));
-    CKI(dalloc(&h->vflag, 4));
-    CKI(dalloc(&h->vinst, ni));
-    {
-      std::vector<int> ones(ni, 1);
-      CKI(cudaMemcpy(h->vinst, ones.data(), sizeof(int) * ni, cudaMemcpyHostToDevice));
-    }
-    const int flags[4] = {1, 1, 0, 0};    // lists invalid until the first build
-    CKI(cudaMemcpy(h->vflag, flags, sizeof(flags), cudaMemcpyHostToDevice));
-    dp.vref = h->vref;
-    dp.vframe = h->vframe;
-    dp.vacc = h->vacc;
+    ws.upload(&h->vacc, std::vector<VAcc>(ni, acc0));
+    ws.upload(&h->vinst, std::vector<int>(ni, 1));
+    ws.upload(&h->vflag, std::vector<int>{1, 1, 0, 0});   // lists invalid until the first build
     // the units as the list kernel's work partition
     h->unit_sched = h->K > 0 ? p->unit_sched : SPH_SCHED_GLOBAL;
     if (h->unit_sched != SPH_SCHED_GLOBAL) {
-      CKI(dalloc(&h->e_of_c, n));
-      CKI(dalloc(&h->perm_e, n));
-      CKI(dalloc(&h->unit_eoff, h->K + 1));
-      CKI(cudaMemset(h->unit_eoff, 0, sizeof(int32_t) * (h->K + 1)));
-      if (p->precision == SPH_PREC_MIXED) CKI(dalloc(reinterpret_cast<float4**>(&h->packAc), n));
-      else CKI(dalloc(reinterpret_cast<D4**>(&h->packAc), n));
-      CKI(dalloc(&h->unit_q, h->K));
-      CKI(dalloc(&h->unit_t, (size_t)2 * h->K));
-      CKI(cudaMemset(h->unit_t, 0, sizeof(unsigned long long) * 2 * h->K));
+      ws.raw(&h->e_of_c, n);
+      ws.raw(&h->perm_e, n);
+      ws.zeroed(&h->unit_eoff, h->K + 1);
+      if (p->precision == SPH_PREC_MIXED) ws.raw(reinterpret_cast<float4**>(&h->packAc), n);
+      else ws.raw(reinterpret_cast<D4**>(&h->packAc), n);
+      ws.raw(&h->unit_q, h->K);
+      ws.zeroed(&h->unit_t, (size_t)2 * h->K);
     }
   }
 
+  h->blocks.push_back(nullptr);
+  CKI(ws.commit(&h->blocks.back(), st));
+  dp.mat = h->mat_dev;
+  dp.slot_org = h->slot_org;
+  dp.vref = h->vref;
+  dp.vframe = h->vframe;
+  dp.vacc = h->vacc;
+
   CKI(launch_check_finite(h, *s, st));
+  unsigned long long* mx = h->counters + 6;               // the largest particle volume (mixed)
+  if (p->precision == SPH_PREC_MIXED) CKI(launch_max_volume(h, *s, mx, st));
   int status = 0;
+  unsigned long long vbits = 0;
+  CKI(cudaMemcpyAsync(&status, h->status, sizeof(int), cudaMemcpyDeviceToHost, st));
+  CKI(cudaMemcpyAsync(&vbits, mx, sizeof(vbits), cudaMemcpyDeviceToHost, st));
   CKI(cudaStreamSynchronize(st));
-  CKI(cudaMemcpy(&status, h->status, sizeof(int), cudaMemcpyDeviceToHost));
   if (status != 0) {
     fail(h, SPH_ERR_NONFINITE, "state holds a non-finite or non-positive value");
     return bail(SPH_ERR_NONFINITE);
@@ -382,14 +401,8 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     // W' wscale ~1 for its smoothing length, which keeps 2 V_i V_j P* W' in the
     // normal FP32 range at any length scale (at 0.1 um spacing V_i V_j ~ 1e-42
     // is below it).  The FP64 rate formation divides them out.
-    unsigned long long* mx = reinterpret_cast<unsigned long long*>(h->counters + 6);
-    CKI(cudaMemsetAsync(mx, 0, sizeof(unsigned long long), st));
-    CKI(launch_max_volume(h, *s, mx, st));
-    unsigned long long bits = 0;
-    CKI(cudaMemcpyAsync(&bits, mx, sizeof(bits), cudaMemcpyDeviceToHost, st));
-    CKI(cudaStreamSynchronize(st));
     double vmax = 0.0;
-    std::memcpy(&vmax, &bits, sizeof(vmax));
+    std::memcpy(&vmax, &vbits, sizeof(vmax));
     if (vmax > 0.0) {
       int ev = 0;
       std::frexp(vmax, &ev);                               // vmax in [2^(ev-1), 2^ev)
@@ -730,6 +743,14 @@ namespace {
 constexpr int kAdjStored = 13;
 constexpr int kAdjW = 16;
 
+// One more block of workspace for the handle.  Where the allocation fails, no pointer is set.
+cudaError_t commit(sph_handle* h, Workspace& ws, cudaStream_t st) {
+  void* base = nullptr;
+  const cudaError_t e = ws.commit(&base, st);
+  if (base) h->blocks.push_back(base);
+  return e;
+}
+
 sph_state adj_work_state(sph_handle* h, const sph_state& ck) {
   const int64_t n = h->n;
   double* w = h->adj_W;
@@ -796,25 +817,35 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
   h->last_stream = st;
   const int64_t n = h->n;
   if (!h->adj_G) {
-    CK(h, dalloc(&h->adj_G, n));
-    CK(h, dalloc(&h->adj_GR, n));
-    CK(h, dalloc(&h->adj_pair, (size_t)11 * n));
-    CK(h, dalloc(&h->adj_par, (size_t)2 * n));
-    CK(h, dalloc(&h->adj_W, (size_t)kAdjW * n));
-    CK(h, cudaMemsetAsync(h->adj_W, 0, sizeof(double) * kAdjW * n, st));
+    Workspace ws;
+    ws.raw(&h->adj_G, n);
+    ws.raw(&h->adj_GR, n);
+    ws.raw(&h->adj_pair, (size_t)11 * n);
+    ws.raw(&h->adj_par, (size_t)2 * n);
+    ws.zeroed(&h->adj_W, (size_t)kAdjW * n);
+    CK(h, commit(h, ws, st));
   }
   // FP64 pair derivatives on a mixed-precision handle (the forward replay stays mixed)
   const bool rev64 = h->dp.precision == SPH_PREC_MIXED && ck->reverse_fp64 != 0;
   if (rev64 && !h->adj64_A) {
-    CK(h, dalloc(reinterpret_cast<D4**>(&h->adj64_A), n));
-    CK(h, dalloc(reinterpret_cast<D4**>(&h->adj64_B), n));
-    CK(h, dalloc(reinterpret_cast<D2**>(&h->adj64_C), n));
-    CK(h, dalloc(&h->adj64_rho, n));
+    Workspace ws;
+    ws.raw(reinterpret_cast<D4**>(&h->adj64_A), n);
+    ws.raw(reinterpret_cast<D4**>(&h->adj64_B), n);
+    ws.raw(reinterpret_cast<D2**>(&h->adj64_C), n);
+    ws.raw(&h->adj64_rho, n);
+    CK(h, commit(h, ws, st));
   }
   if (n_steps > h->adj_store_steps) {
-    if (h->adj_store) CK(h, cudaFree(h->adj_store));
+    if (h->adj_store) {
+      CK(h, cudaFree(h->adj_store));
+      for (void*& p : h->blocks)
+        if (p == h->adj_store) p = nullptr;
+    }
     h->adj_store = nullptr;
-    CK(h, dalloc(&h->adj_store, (size_t)n_steps * kAdjStored * n));
+    h->adj_store_steps = 0;
+    Workspace ws;
+    ws.raw(&h->adj_store, (size_t)n_steps * kAdjStored * n);
+    CK(h, commit(h, ws, st));
     h->adj_store_steps = n_steps;
   }
   sph_state W = adj_work_state(h, ck->state);

@@ -127,6 +127,8 @@ struct sph_handle {
   bool rates_valid = false;
   int steps_since_balance = 0;
 
+  std::vector<void*> blocks;         // device allocations that hold every array below
+
   // segmented blocks: block b covers particles [blk_start[b], blk_end[b]) of instance blk_inst[b]
   int nblk = 0;
   int32_t* blk_inst = nullptr;
@@ -220,12 +222,10 @@ struct sph_handle {
   int vcap = 0;                       // list capacity per particle
   uint32_t* vlist = nullptr;          // [n][vcap]: entry k of slot i at i vcap + k = (slot j << 5) | cell code
   int32_t* vcnt = nullptr;            // [n] entries of slot i
-  double* vref = nullptr;             // [4 n] x, y, z, d of each particle at the last build, then
-                                      // per instance: [6] the frame of the validity criterion (U,
-                                      // steps since the build, U in FP32: 3 floats in the last
-                                      // two), then per instance [4] a VAcc
-  double* vframe = nullptr;           // = vref + 4 n
-  csph::VAcc* vacc = nullptr;         // = vref + 4 n + 6 n_inst (32 bytes each)
+  double* vref = nullptr;             // [4 n] x, y, z, d of each particle at the last build
+  double* vframe = nullptr;           // per instance: [6] the frame of the validity criterion (U, steps
+                                      // since the build, U in FP32: 3 floats in the last two)
+  csph::VAcc* vacc = nullptr;         // [n_inst]
   int* vflag = nullptr;               // [0]: rebuild in this step; [1]: lists invalid; [2]: builds done
   int* vinst = nullptr;               // [n_inst]: instance rebuilt in this step (its mesh, slots and
                                       // lists; the others keep theirs)
