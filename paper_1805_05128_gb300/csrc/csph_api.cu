@@ -782,16 +782,10 @@ cudaError_t copy_dynamic(const sph_state& dst, const sph_state& src, int64_t n, 
   return cudaSuccess;
 }
 
-sph_state stored_state(sph_handle* h, int step, const sph_state& like) {
-  const int64_t n = h->n;
-  double* base = h->adj_store + (size_t)step * kAdjStored * n;
-  sph_state S = like;
-  double** f[kAdjStored] = {&S.x, &S.y, &S.z, &S.vx, &S.vy, &S.vz, &S.rho, &S.E, &S.ax, &S.ay, &S.az, &S.drho,
-                            &S.dE};
-  for (int k = 0; k < kAdjStored; ++k) *f[k] = base + (size_t)k * n;
-  if (h->dp.dim < 2) { S.y = S.vy = S.ay = nullptr; }
-  if (h->dp.dim < 3) { S.z = S.vz = S.az = nullptr; }
-  return S;
+// Between the working state and a stored one: both hold the 13 dynamic arrays
+// side by side, so one copy does (a copy per array was 26 launches per step).
+cudaError_t copy_block(double* dst, const double* src, int64_t n, cudaStream_t st) {
+  return cudaMemcpyAsync(dst, src, sizeof(double) * kAdjStored * n, cudaMemcpyDeviceToDevice, st);
 }
 
 }  // namespace
@@ -852,7 +846,7 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
   // forward replay from the checkpoint with the recorded dt, keeping every state
   CK(h, copy_dynamic(W, ck->state, n, st));
   for (int k = 0; k < n_steps; ++k) {
-    CK(h, copy_dynamic(stored_state(h, k, W), W, n, st));
+    CK(h, copy_block(h->adj_store + (size_t)k * kAdjStored * n, h->adj_W, n, st));
     CK(h, cudaMemcpyAsync(h->dt, ck->dt + k, sizeof(double), cudaMemcpyDeviceToDevice, st));
     CK(h, launch_kick_drift(h, W, st));
     CK(h, launch_build_grid(h, W, st));
@@ -863,15 +857,18 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
   // adjoint, in place in adj_in
   if (adj_in != adj_out) CK(h, copy_dynamic(*adj_in, *adj_out, n, st));
   for (int k = n_steps - 1; k >= 0; --k) {
-    CK(h, copy_dynamic(W, stored_state(h, k, W), n, st));
+    CK(h, copy_block(h->adj_W, h->adj_store + (size_t)k * kAdjStored * n, n, st));
     CK(h, cudaMemcpyAsync(h->dt, ck->dt + k, sizeof(double), cudaMemcpyDeviceToDevice, st));
     CK(h, launch_kick_drift(h, W, st));
-    CK(h, launch_build_grid(h, W, st));
+    // the last step's mesh and packs are still the replay's
+    const bool fresh = k == n_steps - 1;
+    if (!fresh) CK(h, launch_build_grid(h, W, st));
     if (rev64) {
       CK(h, launch_pack_fp64(h, W, true, h->adj64_A, h->adj64_B, h->adj64_C, h->adj64_rho, st));
       CK(h, launch_rates_vjp(h, W, *adj_in, ck->dt + k, 1, adj_params, st, true));
     } else {
-      CK(h, launch_pack(h, W, true, st, false, true));
+      if (fresh) CK(h, cudaMemsetAsync(&h->counters[5], 0, sizeof(unsigned long long), st));   // k_pack's part
+      else CK(h, launch_pack(h, W, true, st, false, true));
       CK(h, launch_rates_vjp(h, W, *adj_in, ck->dt + k, 1, adj_params, st));
     }
   }
