@@ -290,8 +290,7 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
   ws.raw(&h->slot_unit, n);
   if (p->precision == SPH_PREC_MIXED) {
     ws.zeroed(&h->slot_org, (size_t)3 * n);
-    ws.raw(reinterpret_cast<float4**>(&h->packA), n);
-    ws.raw(reinterpret_cast<float4**>(&h->packB), n);
+    ws.raw(reinterpret_cast<float4**>(&h->packA), (size_t)2 * n);   // A and B side by side
     ws.raw(reinterpret_cast<float4**>(&h->packC), n);
   } else {
     ws.raw(reinterpret_cast<D4**>(&h->packA), n);
@@ -352,6 +351,7 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
     h->vcap = (int)std::min(65536.0, std::ceil(cap / 32.0) * 32.0);
     ws.raw(&h->vlist, (size_t)h->vcap * n);
     ws.raw(&h->vcnt, n);
+    if (p->precision == SPH_PREC_MIXED) ws.raw(reinterpret_cast<float4**>(&h->packAc), n);
     const size_t ni = (size_t)n_instances;
     ws.zeroed(&h->vref, (size_t)4 * n);
     // per instance: U = 0 (also its FP32 copy), one step since the build; empty accumulators
@@ -368,8 +368,7 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
       ws.raw(&h->e_of_c, n);
       ws.raw(&h->perm_e, n);
       ws.zeroed(&h->unit_eoff, h->K + 1);
-      if (p->precision == SPH_PREC_MIXED) ws.raw(reinterpret_cast<float4**>(&h->packAc), n);
-      else ws.raw(reinterpret_cast<D4**>(&h->packAc), n);
+      if (p->precision != SPH_PREC_MIXED) ws.raw(reinterpret_cast<D4**>(&h->packAc), n);
       ws.raw(&h->unit_q, h->K);
       ws.zeroed(&h->unit_t, (size_t)2 * h->K);
     }

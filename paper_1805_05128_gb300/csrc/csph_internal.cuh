@@ -155,7 +155,7 @@ struct sph_handle {
   double* slot_org = nullptr;        // mixed: [3 n] cell origin of each cell-order slot (k_cell_sort)
   int32_t* slot_unit = nullptr;      // [n] work unit of slot s
 
-  // packed operands in slot order (FP32 or FP64 by precision)
+  // packed operands in slot order; mixed: A and B of a slot side by side in packA
   void* packA = nullptr;
   void* packB = nullptr;
   void* packC = nullptr;
@@ -239,7 +239,8 @@ struct sph_handle {
   int32_t* e_of_c = nullptr;          // [n] evaluation slot of each cell-order slot
   int32_t* perm_e = nullptr;          // [n] particle of each evaluation slot
   int32_t* unit_eoff = nullptr;       // [K + 1] start of each unit's evaluation range
-  void* packAc = nullptr;             // [n] cell-order copy of the position / size operand (list build)
+  void* packAc = nullptr;             // [n] cell-order copy of the position / size operand (list build;
+                                      // mixed handles with lists, and unit schedules)
   unsigned long long* unit_q = nullptr;   // [K] per-unit work counters of the list kernel
   unsigned long long* unit_t = nullptr;   // [2K] first group start and last group end per unit (ns)
 

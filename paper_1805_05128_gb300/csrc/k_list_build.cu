@@ -47,8 +47,8 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   const int64_t total = *a.total_cells_dev;
-  // the cell-order copy of the positions when the lists are laid out in the
-  // unit-major evaluation order
+  // positions and sizes in cell order: k_pack's copy (mixed handles, whose packs
+  // hold B beside A, and unit-major evaluation orders), else the pack itself
   const V4* __restrict__ A = reinterpret_cast<const V4*>(a.Ac ? a.Ac : a.A);
   // Persistent warps: each takes the next cell from a global counter, so the
   // work spreads evenly whatever the mix of empty and crowded cells.
@@ -261,10 +261,8 @@ cudaError_t launch_list_build(sph_handle* h, const sph_state& s, cudaStream_t st
   const double khl = h->dp.kh * (1.0 + h->dp.cell_beta);
   a.kh = khl;
   a.kh_f = (float)khl;
-  if (h->unit_sched != SPH_SCHED_GLOBAL) {   // rows and entries in the unit-major evaluation order
-    a.e_of_c = h->e_of_c;
-    a.Ac = h->packAc;
-  }
+  if (h->unit_sched != SPH_SCHED_GLOBAL) a.e_of_c = h->e_of_c;   // rows and entries in the unit-major evaluation order
+  a.Ac = h->packAc;                                               // A alone, in cell order
   // work counter zeroed by the step's k_pack
   a.work_counter = &h->counters[7];
   a.vinst = h->n_inst > 1 ? h->vinst : nullptr;   // only the instances whose lists are rebuilt

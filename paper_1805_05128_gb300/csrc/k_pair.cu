@@ -76,7 +76,6 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
   const unsigned lt = (1u << lane) - 1u;
   const int home = lane / G, hl = lane % G;                   // the lane's slot in the group, its place in the slot
   const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
-  const V4* __restrict__ B = reinterpret_cast<const V4*>(a.B);
   const VC* __restrict__ C = reinterpret_cast<const VC*>(a.C);
   // Persistent warps: the first group of each is fixed (spread over the CTAs,
   // so that few groups run on many SMs), the following ones come from a
@@ -105,11 +104,11 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
       row = lc / g.dims[0];
       cx = lc - row * g.dims[0];
     }
-    const V4 Ai = A[ii];
+    V4 Ai, Bi;
+    load_AB(a.A, a.B, (uint32_t)ii, Ai, Bi);
     int cnt = 0, seg_of = 0, cx_seg = 0;
     unsigned nfull = 0, ncand = 0, nexact = 0;
     const int ui = a.K > 0 ? a.slot_unit[ii] : 0;
-    const V4 Bi = B[ii];
     const VC Ci = C[ii];
     // reverse mode: i's adjoint operands and the 11 own-side sums
     const V4* __restrict__ Gp = reinterpret_cast<const V4*>(a.G);
@@ -135,8 +134,8 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
     auto grad_terms = [&](int64_t j, T sx, T sy, T sz) -> GradTerms {
       GradTerms q{};
       if (j == i) return q;
-      const V4 Aj = A[j];
-      const V4 Bj = B[j];
+      V4 Aj, Bj;
+      load_AB(a.A, a.B, (uint32_t)j, Aj, Bj);
       const VC Cj = C[j];
       T dx, dy, dz;
       if (MIXED) {
@@ -190,8 +189,8 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
     // V = m/rho, d (through h_ij) and the rho factor of the continuity term.
     auto pair_vjp = [&](int64_t j, T sx, T sy, T sz) {
       if (j == i) return;
-      const V4 Aj = A[j];
-      const V4 Bj = B[j];
+      V4 Aj, Bj;
+      load_AB(a.A, a.B, (uint32_t)j, Aj, Bj);
       const VC Cj = C[j];
       const V4 Gj = Gp[j];
       const V2 Rj = Rp[j];
@@ -512,7 +511,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
           const bool jv = j < r1;
           const int jl = jv ? j : r0;
           const int relx = a.slot_cell[jl] - (int)rb - cx0;
-          const float4 S = frame(A[jl], relx, oy, oz);
+          const float4 S = frame(load_A(A, jl), relx, oy, oz);
           // keep the candidates within reach of the members' box (a superset:
           // every rounding below is monotone in the distance)
           const float gx = fmaxf(0.f, fmaxf(S.x - bxh, bxl - S.x));

@@ -88,7 +88,6 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = lane / kSlotLanes, hl = lane % kSlotLanes;   // the slot's group of lanes, lane in it
-  const V4* __restrict__ A = reinterpret_cast<const V4*>(a.A);
   // Work partition.  SPH_SCHED_GLOBAL: groups of 32 consecutive slots from one
   // global counter, the last ones of 8 (launch_lists_one).  Units: each unit owns a contiguous range of evaluation
   // slots and a counter; CTA b starts on unit b K / gridDim.x (the CTAs are
@@ -173,15 +172,14 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
     // is in bounds.
     uint32_t e_pre = 0u, e_pre1 = 0u;
     int cnt_pre = 0;
-    const V4* __restrict__ Bp = reinterpret_cast<const V4*>(a.B);
     const VC* __restrict__ Cp = reinterpret_cast<const VC*>(a.C);
     int stage = 0;
     // STAGE: copy the operands of entry e (or of slot `self`, a stand-in that
     // accepts nothing, for a lane without an entry) into stage st
     auto stage_ops = [&](int st, bool has, uint32_t e, int self) {
       const int64_t j = has ? (int64_t)(e >> 5) : (int64_t)self;
-      const char* ga = reinterpret_cast<const char*>(A + j);
-      const char* gb = reinterpret_cast<const char*>(Bp + j);
+      const char* ga = reinterpret_cast<const char*>(a.A) + 2 * sizeof(V4) * j;   // A, then B
+      const char* gb = ga + sizeof(V4);
       const char* gc = reinterpret_cast<const char*>(Cp + j);
 #pragma unroll
       for (int c = 0; c < kChA; ++c) cp16(&stg[warp][st][c][lane], ga + 16 * c);
@@ -230,8 +228,8 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       const GridInfo& g = a.grid[b];
       const T dcs = MIXED ? (T)g.dc_f : T(0);
       const float band = MIXED ? 0x1p-12f * g.dc_f * g.dc_f : 0.f;
-      const V4 Ai = A[ii];
-      const V4 Bi = Bp[ii];
+      V4 Ai, Bi;
+      load_AB(a.A, a.B, (uint32_t)ii, Ai, Bi);
       const VC Ci = Cp[ii];
       const T khdi = MIXED ? (T)a.kh_f * Ai.w : T(0);
       const int ui = a.K > 0 ? a.slot_unit[ii] : 0;
@@ -314,7 +312,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
             const uint32_t e = kv ? e_cur : 0u;
             e_cur = row[k + kSlotLanes < a.vcap ? k + kSlotLanes : k];
             const uint32_t j = e >> 5;
-            const V4 Aj = A[j];
+            const V4 Aj = reinterpret_cast<const V4*>(a.A)[j];
             const float tx = f32_scaled(Aj.x - Ai.x, ex);
             const float ty = DIM >= 2 ? f32_scaled(Aj.y - Ai.y, ex) : 0.f;
             const float tz = DIM >= 3 ? f32_scaled(Aj.z - Ai.z, ex) : 0.f;

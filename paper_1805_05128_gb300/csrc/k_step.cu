@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_pack(DevParams P, sph_state s, co
     for (int a = 0; a < 3; ++a)
       if (a < P.dim) off[a] = f32_rn(X[a] - P.slot_org[(int64_t)a * P.n + sc]);
     const float4 Arec = make_float4(off[0], off[1], off[2], f32_rn(d));
-    reinterpret_cast<float4*>(packA)[sl] = Arec;
+    reinterpret_cast<float4*>(packA)[2 * sl] = Arec;
     if (build) reinterpret_cast<float4*>(packAc)[sc] = Arec;
     const float Vp = fast ? (f32_rn(m) / f32_rn(rho)) * P.vscale_f : (float)((m / rho) * P.vscale);
     // FP32 velocities relative to a reference velocity of whole m/s per
@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_pack(DevParams P, sph_state s, co
     for (int a = 0; a < 3; ++a)
       if (a < P.dim) vr[a] = f32_rn(v[a] - trunc_ref(v[a], k[a]));
     const uint32_t kxy = (uint32_t)(k[0] + 32768) | ((uint32_t)(k[1] + 32768) << 16);
-    reinterpret_cast<float4*>(packB)[sl] = make_float4(vr[0], vr[1], vr[2], Vp);
+    reinterpret_cast<float4*>(packA)[2 * sl + 1] = make_float4(vr[0], vr[1], vr[2], Vp);
     reinterpret_cast<float4*>(packC)[sl] = make_float4(f32_rn(Pp), fast ? f32_rn(rho) * cf : (float)(rho * cp),
                                                        __uint_as_float(kxy), (float)k[2]);
   } else {
@@ -1041,7 +1041,7 @@ cudaError_t launch_pack(sph_handle* h, const sph_state& s, bool predict, cudaStr
   const int kc = keep_counts ? 1 : 0;
   const int32_t* eoc = eorder ? h->e_of_c : nullptr;
   int32_t* pe = eorder ? h->perm_e : nullptr;
-  void* Ac = eorder ? h->packAc : nullptr;
+  void* Ac = h->packAc;   // written only when a list build follows
   if (h->dp.precision == SPH_PREC_MIXED)
     CKL(launch_chained(k_pack<true>, dim3(h->nblk), dim3(kBlock), st, h->dp, s, h->blk_start, h->blk_end, h->blk_inst, h->grid, h->dt,
                                              predict ? 1 : 0, h->perm, h->cell_of, h->packA, h->packB, h->packC,
