@@ -347,34 +347,11 @@ __global__ void k_scan_reduce(const int32_t* __restrict__ cnt, const int64_t* __
   }
 }
 
-// Single block: exclusive scan of the tile sums in place.
-__global__ void k_scan_sums(int32_t* sums, const int64_t* __restrict__ total, const int* __restrict__ gate) {
-  chain_entry();
-  if (gate && gate[0] == 0) return;   // Verlet mode: mesh kept from the last build
-  int64_t ntiles = (*total + kScanTile - 1) / kScanTile;
-  __shared__ int carry;
-  __shared__ int sh[1024];
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int64_t base = 0; base < ntiles; base += blockDim.x) {
-    int64_t i = base + threadIdx.x;
-    int v = (i < ntiles) ? sums[i] : 0;
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-      int add = threadIdx.x >= (unsigned)off ? sh[threadIdx.x - off] : 0;
-      __syncthreads();
-      sh[threadIdx.x] += add;
-      __syncthreads();
-    }
-    if (i < ntiles) sums[i] = carry + sh[threadIdx.x] - v;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry += sh[threadIdx.x];
-    __syncthreads();
-  }
-}
-
 // Per tile: exclusive scan plus tile offset; zero the counts for the next use.
+// A block adds up the sums of the tiles before its own itself (4 bytes of L2
+// per 1024 cells): a one-block scan of them between the two kernels cost a
+// launch and its latency per mesh build (400-particle FP64 tube with a mesh per
+// step: 1123 -> 1065 us a pass; 32k plate impact with lists: 553 -> 544).
 __global__ void k_scan_down(int32_t* cnt, const int64_t* __restrict__ total, const int32_t* __restrict__ sums,
                             int32_t* start, int64_t n_total, const int* __restrict__ gate) {
   chain_entry();
@@ -382,8 +359,18 @@ __global__ void k_scan_down(int32_t* cnt, const int64_t* __restrict__ total, con
   const int64_t tot = *total;
   constexpr int per = kScanTile / kBlock;  // 4 cells per thread
   __shared__ int sh[kBlock];
+  __shared__ int wsum[kBlock / 32];
+  int64_t before = 0;                       // tiles whose sums are in `offset`
+  int offset = 0;
   for (int64_t t = blockIdx.x; t * kScanTile < tot; t += gridDim.x) {
     const int64_t base = t * kScanTile;
+    int part = 0;
+    for (int64_t k = before + threadIdx.x; k < t; k += blockDim.x) part += sums[k];
+    part = __reduce_add_sync(0xffffffffu, part);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = part;
+    __syncthreads();
+    for (int w = 0; w < kBlock / 32; ++w) offset += wsum[w];
+    before = t;
     int vals[per];
     int run = 0;
     for (int k = 0; k < per; ++k) {
@@ -399,7 +386,7 @@ __global__ void k_scan_down(int32_t* cnt, const int64_t* __restrict__ total, con
       sh[threadIdx.x] += add;
       __syncthreads();
     }
-    int acc = sums[t] + sh[threadIdx.x] - run;
+    int acc = offset + sh[threadIdx.x] - run;
     for (int k = 0; k < per; ++k) {
       int64_t c = base + threadIdx.x * per + k;
       if (c < tot) {
@@ -1026,11 +1013,10 @@ cudaError_t launch_build_grid(sph_handle* h, const sph_state& s, cudaStream_t st
   CKL(launch_chained(k_cell_count, dim3(capped_grid(h->nblk)), dim3(kBlock), st, a));
   int tiles = capped_grid(grid_for(h->cell_cap, kScanTile));
   CKL(launch_chained(k_scan_reduce, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, gate));
-  CKL(launch_chained(k_scan_sums, dim3(1), dim3(1024), st, h->scan_sums, h->total_cells, gate));
   CKL(launch_chained(k_scan_down, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, h->cell_start, h->n, gate));
   CKL(launch_chained(k_cell_scatter, dim3(capped_grid(grid_for(h->n, kBlock))), dim3(kBlock), st, a));
   CKL(launch_chained(k_cell_sort, dim3(capped_grid(grid_for(h->cell_cap * 32, kBlock))), dim3(kBlock), st, a));
-  h->launches += 6;
+  h->launches += 5;
   // a mesh built outside the Verlet sequence changes the slot order under the lists
   if (!gate && h->verlet) return cudaMemsetAsync(&h->vflag[1], 0xff, sizeof(int), st);
   return cudaGetLastError();
@@ -1127,11 +1113,10 @@ cudaError_t launch_exclusive_scan(int32_t* cnt, const int64_t* total, int32_t* s
                                   int64_t n_total, int64_t cap, cudaStream_t st, const int* gate) {
   int tiles = capped_grid(grid_for(cap, kScanTile));
   k_scan_reduce<<<tiles, kBlock, 0, st>>>(cnt, total, sums, gate);
-  k_scan_sums<<<1, 1024, 0, st>>>(sums, total, gate);
   k_scan_down<<<tiles, kBlock, 0, st>>>(cnt, total, sums, start, n_total, gate);
   return cudaGetLastError();
 }
-// (launch_exclusive_scan's three kernels are counted by its callers)
+// (launch_exclusive_scan's two kernels are counted by its callers)
 
 cudaError_t launch_conservation(sph_handle* h, const sph_state& s, double* out, cudaStream_t st) {
   const int per = cluster_size_for(k_conservation, kSumBlock, h->n / h->n_inst, 4096);

@@ -536,7 +536,7 @@ cudaError_t launch_unit_lists(sph_handle* h, const int32_t* unit, int32_t* unit_
   if (e != cudaSuccess) return e;
   k_unit_scatter<<<nb, kUnitBlock, smem, st>>>(unit, h->n, K, nb, starts, h->unit_list);
   k_unit_offsets<<<grid_for(K + 1, kBlock), kBlock, 0, st>>>(starts, K, nb, h->n, h->unit_off, unit_offsets);
-  h->launches += 6;
+  h->launches += 5;
   return cudaGetLastError();
 }
 
@@ -589,7 +589,7 @@ cudaError_t launch_eorder(sph_handle* h, const sph_state& s, cudaStream_t st, bo
   k_unit_scatter<<<nb, kUnitBlock, smem, st>>>(slot_u, h->n, K, nb, starts, c_of_e, gate);
   k_unit_offsets<<<grid_for(K + 1, kBlock), kBlock, 0, st>>>(starts, K, nb, h->n, h->unit_eoff, nullptr, gate);
   k_eorder_inverse<<<g, kBlock, 0, st>>>(h->n, c_of_e, h->perm, h->e_of_c, h->perm_e, gate);
-  h->launches += 8;
+  h->launches += 7;
   return cudaGetLastError();
 }
 
