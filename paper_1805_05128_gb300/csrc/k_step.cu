@@ -61,47 +61,67 @@ __device__ __forceinline__ void red_merge(Red& a, const Red& b) {
   a.viol = a.viol > b.viol ? a.viol : b.viol;
 }
 
-__device__ __forceinline__ Red shfl_red(const Red& r, int o) {
-  Red q;
-  for (int a = 0; a < 3; ++a) {
-    q.lo[a] = __shfl_xor_sync(0xffffffffu, r.lo[a], o);
-    q.hi[a] = __shfl_xor_sync(0xffffffffu, r.hi[a], o);
-    q.dlo[a] = __shfl_xor_sync(0xffffffffu, r.dlo[a], o);
-    q.dhi[a] = __shfl_xor_sync(0xffffffffu, r.dhi[a], o);
-  }
-  q.d1 = __shfl_xor_sync(0xffffffffu, r.d1, o);
-  q.d2 = __shfl_xor_sync(0xffffffffu, r.d2, o);
-  q.viol = __shfl_xor_sync(0xffffffffu, r.viol, o);
-  return q;
+// Minimum / maximum of a 64-bit key over a full warp: the signed high word,
+// then the low word among the lanes that hold it, two redux instructions
+// where a butterfly takes ten shuffles and five 64-bit compares.
+__device__ __forceinline__ long long warp_min(long long k) {
+  const int hi = (int)(k >> 32), m = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_min_sync(0xffffffffu, hi == m ? (unsigned)k : 0xffffffffu);
+  return (long long)(((unsigned long long)(unsigned)m << 32) | lo);
 }
 
-// Block-wide reduction of Red: butterfly within each warp, then the warp
-// results through shared memory; result in thread 0.  Every merge is a
-// min / max / top-2 of integer keys, so the order does not change the result.
-__device__ void block_reduce(Red& r) {
-  __shared__ Red sh[kBlock / 32];
+__device__ __forceinline__ long long warp_max(long long k) {
+  const int hi = (int)(k >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)k : 0u);
+  return (long long)(((unsigned long long)(unsigned)m << 32) | lo);
+}
+
+// The two largest sizes: the largest d1, then that lane's d2 against the other
+// lanes' d1.  The Verlet keys stay as they are without `verlet` (a kernel
+// without a list handle leaves them at red_init).
+__device__ __forceinline__ void warp_reduce(Red& r, int dim, bool verlet) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) red_merge(r, shfl_red(r, o));
+  for (int a = 0; a < 3; ++a)
+    if (a < dim) {
+      r.lo[a] = warp_min(r.lo[a]);
+      r.hi[a] = warp_max(r.hi[a]);
+      if (verlet) {
+        r.dlo[a] = __reduce_min_sync(0xffffffffu, r.dlo[a]);
+        r.dhi[a] = __reduce_max_sync(0xffffffffu, r.dhi[a]);
+      }
+    }
+  const long long m = warp_max(r.d1);
+  const int first = __ffs(__ballot_sync(0xffffffffu, r.d1 == m)) - 1;
+  r.d2 = warp_max((int)(threadIdx.x & 31) == first ? r.d2 : r.d1);
+  r.d1 = m;
+  if (verlet) r.viol = warp_max(r.viol);
+}
+
+// Block-wide reduction of Red, once per kernel: each warp, then the first warp
+// over the warps' results; result in thread 0.  Every merge is a min / max /
+// top-2 of integer keys, so the order does not change the result.  (With
+// butterflies and one thread merging the warps it was half of the kick-drift's
+// 996 instructions a warp.)
+__device__ void block_reduce(Red& r, int dim, bool verlet) {
+  __shared__ Red sh[kBlock / 32];
+  warp_reduce(r, dim, verlet);
   const int t = threadIdx.x;
   if ((t & 31) == 0) sh[t >> 5] = r;
   __syncthreads();
-  if (t == 0)
-    for (int w = 1; w < kBlock / 32; ++w) red_merge(r, sh[w]);
-  __syncthreads();
+  if (t < 32) {
+    if (t < (int)(blockDim.x >> 5)) r = sh[t];
+    else red_init(r);
+    warp_reduce(r, dim, verlet);
+  }
 }
 
 // Block minimum of the dt keys only (a step's k_derive); result in thread 0.
 __device__ long long block_min_key(long long k) {
   __shared__ long long sh[kBlock / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long q = __shfl_xor_sync(0xffffffffu, k, o);
-    k = q < k ? q : k;
-  }
+  k = warp_min(k);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int w = 1; w < kBlock / 32; ++w) k = sh[w] < k ? sh[w] : k;
+  if (threadIdx.x < 32) k = warp_min(threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : LLONG_MAX);
   return k;
 }
 
@@ -136,7 +156,7 @@ __global__ void k_derive(DevParams P, sph_state s, const int64_t* __restrict__ b
     if (P.dim >= 3) r.lo[2] = r.hi[2] = dkey(s.z[p]);
     r.d1 = dkey(d);
   }
-  block_reduce(r);
+  block_reduce(r, P.dim, false);
   if (threadIdx.x == 0) write_part(part, r);
 }
 
@@ -196,7 +216,7 @@ __device__ void mesh_reduce_inst(int b, const int32_t* inst_blk, const BlockPart
     q.d1 = part[k].d1; q.d2 = part[k].d2;
     red_merge(r, q);
   }
-  block_reduce(r);
+  block_reduce(r, 3, false);
   if (threadIdx.x == 0) {
     GridInfo& g = grid[b];
     for (int a = 0; a < 3; ++a) { g.x0[a] = dunkey(r.lo[a]); g.hi[a] = dunkey(r.hi[a]); }
@@ -674,7 +694,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_kick_drift(DevParams P, sph_state
     }
     if (!finite || !finite_bits(d)) set_status(status, SPH_ERR_NONFINITE);
   }
-  block_reduce(r);
+  block_reduce(r, P.dim, P.vref != nullptr);
   if (threadIdx.x == 0) {
     write_part(part, r);
     if (P.vacc) {                  // the criterion's maximum and displacement box of the instance
@@ -742,9 +762,12 @@ __global__ void k_kick2(DevParams P, sph_state s, const int64_t* __restrict__ bl
 //          cell origin o, the local-origin idea of Sec. 3.1), B = {v, m/rho},
 //          C = {P, rho c}
 //   fp64 : A = {x, y, z, d} (global positions), B, C in FP64
+// Bound by the latency of its gathers (FP64 pipe 62 %, DRAM 43 % of peak at
+// 1.125M), so mixed runs 6 blocks an SM although that spills a few words: five
+// steps of the 1.125M plate impact with lists 5405 / 5376 / 5345 us at 4 / 5 / 6.
 // ---------------------------------------------------------------------------
 template <bool MIXED>
-__global__ void __launch_bounds__(kBlock, 4) k_pack(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
+__global__ void __launch_bounds__(kBlock, MIXED ? 6 : 4) k_pack(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
                        const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst,
                        const GridInfo* __restrict__ grid, const double* __restrict__ dt, int predict,
                        const int32_t* __restrict__ perm, const int32_t* __restrict__ cell_of,
