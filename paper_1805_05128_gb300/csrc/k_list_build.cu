@@ -6,40 +6,53 @@
 // cell of edge (1 + beta) D^c holds 27 particles of a lattice, so a warp per
 // cell fills its lanes here).  For each neighbour row (the 3 x-consecutive
 // cells at (oy, oz), contiguous in slot order) each lane loads one candidate;
-// those within reach of the home group's bounding box are compacted into
-// shared memory in order, and every lane tests its own home particle against
-// each (a broadcast read) and appends the accepted ones to its row in
-// candidate order.  A row entry is 16 bits: the neighbour-cell code (ox+1) +
-// 3 (oy+1) + 9 (oz+1) and the offset inside that cell.  The warp then writes
-// each home particle's row with 32 consecutive stores.
+// those within reach of the home group's bounding box enter a queue in shared
+// memory, in order.  Whenever the queue holds 32, every lane tests its own
+// home particle against each (broadcast reads, two candidates per packed FP32
+// operation) into a bit mask, and the warp writes, home particle by home
+// particle, the entries of the set bits to consecutive places of its row: lane
+// c holds candidate c's entry, (slot j << 5) | (ox+1) + 3 (oy+1) + 9 (oz+1).
 //
 // The test runs in FP32 in both precisions (mixed handles on the packed
 // offsets from the cell origins, FP64 handles on offsets from the cell's first
 // particle scaled to a cell edge of ~1) and accepts r^2 - R^2 < 2^-12 D^c^2, a
-// superset of the radius: k_pair_lists decides each entry exactly.  Bound by
-// shared-memory latency and issue.
+// superset of the radius: k_pair_lists decides each entry exactly.
+// Bound by issue (77 % of the slots) and the latency of its short phases:
+// 659 us at 1.125M particles, 768 us at 1M droplet particles.  Rows gathered in
+// shared memory, one append per test and lane, and flushed at the end (33 KB a
+// block, scalar tests, 68 % of the issue slots): 740 and 854 us.
 #include "pair_common.cuh"
 
 namespace csph {
 
 namespace {
 
-// Row capacity between flushes and resident blocks per SM: rows of 64 or 96
-// entries with 7-8 resident blocks made the 1.125M plate's step 0.3-3 % slower
-// than 128 entries with 6 blocks.  Row stride: cap + 2 16-bit entries, an odd
-// number of words, so lane rows fall in distinct banks.
-constexpr int kBuildCap = 128;
-constexpr int kBuildBlocks = 6;
+constexpr int kQueue = 64;         // under 32 waiting candidates and a chunk of 32
 
+// Minimum / maximum over a full warp (one redux instruction; a NaN loses).
+__device__ __forceinline__ float warp_min(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// Resident blocks: mixed 8 / 7 / 6 took 5305 / 5212 / 5230 us for five steps of
+// the 1.125M plate impact; FP64 7 / 6 took 1676 / 1657 us for two of a 65k ejecta cloud.
 template <bool MIXED, int DIM>
-__global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArgs a) {
+__global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairArgs a) {
   chain_entry();
   using T = typename Ops<MIXED>::T;
   using V4 = typename Ops<MIXED>::V4;
   using F = Pair<true, DIM>;
-  __shared__ uint16_t list[kWarps][32][kBuildCap + 2];      // [warp][home particle][entry]
-  __shared__ float4 cand[kWarps][32];                        // candidates: x, y, z in the home cell's frame, d
-  __shared__ uint16_t cand_ent[kWarps][32];                  // their list entries
+  // the queue, component by component: x, y, z in the home cell's frame, d
+  __shared__ alignas(16) float qx[kWarps][kQueue], qy[kWarps][kQueue], qz[kWarps][kQueue], qd[kWarps][kQueue];
+  __shared__ uint32_t qword[kWarps][kQueue];                 // the entry of a row
+  __shared__ int32_t qslot[kWarps][kQueue];                  // the candidate's slot in cell order
   __shared__ int32_t nb_start[kWarps][27];                   // start slot of each neighbour cell
 
   if (a.vflag[0] == 0) return;                               // lists still valid: nothing to build
@@ -115,45 +128,72 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
       const int ii = act ? i : hs;
       const float4 H = frame(A[ii], 0, 0, 0);
       const float khdi = a.kh_f * H.w;
-      int cnt = 0, vc = 0;
+      const int row_i = a.e_of_c ? a.e_of_c[ii] : ii;        // the row's slot
+      int vc = 0;
       // the home group's bounding box and largest kh d, a warp-wide cull of candidates
-      float bxl = H.x, bxh = H.x, byl = H.y, byh = H.y, bzl = H.z, bzh = H.z, bkh = khdi;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        bxl = fminf(bxl, __shfl_xor_sync(0xffffffffu, bxl, o)); bxh = fmaxf(bxh, __shfl_xor_sync(0xffffffffu, bxh, o));
-        byl = fminf(byl, __shfl_xor_sync(0xffffffffu, byl, o)); byh = fmaxf(byh, __shfl_xor_sync(0xffffffffu, byh, o));
-        bzl = fminf(bzl, __shfl_xor_sync(0xffffffffu, bzl, o)); bzh = fmaxf(bzh, __shfl_xor_sync(0xffffffffu, bzh, o));
-        bkh = fmaxf(bkh, __shfl_xor_sync(0xffffffffu, bkh, o));
-      }
+      const float bxl = warp_min(H.x), bxh = warp_max(H.x), byl = warp_min(H.y), byh = warp_max(H.y);
+      const float bzl = warp_min(H.z), bzh = warp_max(H.z), bkh = warp_max(khdi);
+      int head = 0, tail = 0;                                // of the queue (warp-uniform); head a multiple of 32
 
-      // The warp writes each home particle's new entries together, 32
-      // consecutive entries of one row per store (the self pair dropped by a
-      // ballot, list order kept), instead of one entry of 32 rows per store.
-      auto flush_lists = [&]() {
-        for (int hp = 0; hp < nh; ++hp) {
-          const int n = __shfl_sync(0xffffffffu, cnt, hp);
-          int v0 = __shfl_sync(0xffffffffu, vc, hp);
-          const int64_t ih = a.e_of_c ? (int64_t)a.e_of_c[h0 + hp] : (int64_t)(h0 + hp);   // the row's slot
-          const int64_t ihc = h0 + hp;                                                       // cell order
-          for (int k0 = 0; k0 < n; k0 += 32) {
-            const int k = k0 + lane;
-            uint32_t word = 0;
-            bool w = false;
-            if (k < n) {
-              const unsigned ent = list[warp][hp][k];
-              const int64_t j = (int64_t)nb_start[warp][ent >> 11] + (ent & 2047u);
-              w = j != ihc;
-              const int64_t je = a.e_of_c ? (int64_t)a.e_of_c[j] : j;
-              word = ((uint32_t)je << 5) | (ent >> 11);
+      // the test of the first nc (at most 32) queued candidates, and their entries
+      auto drain = [&](int nc) {
+        const int at = head & (kQueue - 1);
+        const float2 nx2 = make_float2(-H.x, -H.x), ny2 = make_float2(-H.y, -H.y), nz2 = make_float2(-H.z, -H.z);
+        const float2 kh2 = make_float2(a.kh_f, a.kh_f), kd2 = make_float2(khdi, khdi);
+        const float2 nk2 = make_float2(-a.kh_f, -a.kh_f), nd2 = make_float2(-khdi, -khdi);
+        unsigned mask = 0;
+#pragma unroll
+        for (int c = 0; c < 32; c += 4) {
+          if (c >= nc) break;
+          const float4 X = *reinterpret_cast<const float4*>(&qx[warp][at + c]);
+          const float4 D = *reinterpret_cast<const float4*>(&qd[warp][at + c]);
+          float4 Y{}, Z{};
+          if (DIM >= 2) Y = *reinterpret_cast<const float4*>(&qy[warp][at + c]);
+          if (DIM >= 3) Z = *reinterpret_cast<const float4*>(&qz[warp][at + c]);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const float2 dx = add2(k ? make_float2(X.z, X.w) : make_float2(X.x, X.y), nx2);
+            float2 r2 = mul2(dx, dx);
+            if (DIM >= 2) {
+              const float2 dy = add2(k ? make_float2(Y.z, Y.w) : make_float2(Y.x, Y.y), ny2);
+              r2 = fma2(dy, dy, r2);
             }
-            const unsigned m = __ballot_sync(0xffffffffu, w);
-            const int pos = v0 + __popc(m & lt);
-            if (w && pos < a.vcap) a.vlist[ih * a.vcap + pos] = word;
-            v0 += __popc(m);
+            if (DIM >= 3) {
+              const float2 dz = add2(k ? make_float2(Z.z, Z.w) : make_float2(Z.x, Z.y), nz2);
+              r2 = fma2(dz, dz, r2);
+            }
+            const float2 d = k ? make_float2(D.z, D.w) : make_float2(D.x, D.y);
+            const float2 diff = fma2(fma2(nk2, d, nd2), fma2(kh2, d, kd2), r2);   // r^2 - R^2
+            if (diff.x < band) mask |= 1u << (c + 2 * k);
+            if (diff.y < band) mask |= 2u << (c + 2 * k);
           }
-          if (lane == hp) vc = v0;
         }
-        cnt = 0;
+        if (nc < 32) mask &= (1u << nc) - 1u;
+        if (!act) mask = 0;
+        const bool mine = lane < nc;
+        const int jc = mine ? qslot[warp][at + lane] : -1;
+        const uint32_t word = mine ? qword[warp][at + lane] : 0u;
+        // no pair with itself: the home particles in this chunk are consecutive candidates
+        const unsigned own = __ballot_sync(0xffffffffu, jc >= h0 && jc < h0 + nh);
+        if (own) {
+          const int first = __ffs(own) - 1;
+          const unsigned k = (unsigned)(i - __shfl_sync(0xffffffffu, jc, first));
+          if (k < (unsigned)__popc(own)) mask &= ~(1u << (first + k));
+        }
+        for (int h8 = 0; h8 < nh; h8 += 8) {   // (the masks of lanes past nh are empty)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int hp = h8 + k;
+            const unsigned m = __shfl_sync(0xffffffffu, mask, hp);
+            const int v0 = __shfl_sync(0xffffffffu, vc, hp);
+            const int row = a.e_of_c ? __shfl_sync(0xffffffffu, row_i, hp) : h0 + hp;
+            const int pos = v0 + __popc(m & lt);
+            if (((m >> lane) & 1u) && pos < a.vcap) a.vlist[(int64_t)row * a.vcap + pos] = word;
+          }
+        }
+        vc += __popc(mask);
+        head += nc;
+        __syncwarp();   // the places read are written again by the next chunks
       };
 
       for (int oz = (DIM >= 3 ? -1 : 0); oz <= (DIM >= 3 ? 1 : 0); ++oz) {
@@ -168,8 +208,6 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
           const int r1 = a.cell_start[rowc + xe];
           const int b1 = a.cell_start[rowc + cx + 1];      // end of the ox = 0 cell
           for (int base = r0; base < r1; base += 32) {
-            // a chunk adds at most 32 entries to a list: flush first if one could overflow
-            if (__any_sync(0xffffffffu, cnt > kBuildCap - 32)) flush_lists();
             const int j = base + lane;
             const bool jv = j < r1;
             const V4 R = A[jv ? j : r0];
@@ -180,7 +218,7 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
               S = frame(R, ox, oy, oz);
               const int off = j - (ox < 0 ? s_m : (ox == 0 ? s_0 : b1));
               if (off > 2047) set_status(a.status, SPH_ERR_CAPACITY);   // cell over 2047 particles
-              ent = ((uint32_t)(rc + ox + 1) << 11) | (uint32_t)(off & 2047);
+              ent = ((uint32_t)(a.e_of_c ? a.e_of_c[j] : j) << 5) | (uint32_t)(rc + ox + 1);
             }
             // keep only the candidates within reach of the home group's box
             // (a superset: every rounding below is monotone in the distance)
@@ -191,28 +229,24 @@ __global__ void __launch_bounds__(kPairBlock, kBuildBlocks) k_list_build(PairArg
             const bool keep = jv && fmaf(-Rm, Rm, F::r2_of(gx, gy, gz)) < band;
             const unsigned km = __ballot_sync(0xffffffffu, keep);
             if (keep) {
-              const int c = __popc(km & lt);
-              cand[warp][c] = S;
-              cand_ent[warp][c] = (uint16_t)ent;
+              const int c = (tail + __popc(km & lt)) & (kQueue - 1);
+              qx[warp][c] = S.x;
+              if (DIM >= 2) qy[warp][c] = S.y;
+              if (DIM >= 3) qz[warp][c] = S.z;
+              qd[warp][c] = S.w;
+              qword[warp][c] = ent;
+              qslot[warp][c] = j;
             }
-            const int nc = __popc(km);
+            tail += __popc(km);
             __syncwarp();
-#pragma unroll 8
-            for (int c = 0; c < nc; ++c) {
-              const float4 Sc = cand[warp][c];
-              const float r2 = F::r2_of(Sc.x - H.x, DIM >= 2 ? Sc.y - H.y : 0.f, DIM >= 3 ? Sc.z - H.z : 0.f);
-              const float R = fmaf(a.kh_f, Sc.w, khdi);
-              const float diff = fmaf(-R, R, r2);          // r^2 - R^2
-              if (diff < band && act) list[warp][lane][cnt++] = cand_ent[warp][c];
-            }
-            __syncwarp();   // the candidate buffer is rewritten by the next chunk
+            if (tail - head >= 32) drain(32);
           }
         }
       }
-      flush_lists();
+      if (tail > head) drain(tail - head);
       if (act) {
         if (vc > a.vcap) set_status(a.status, SPH_ERR_CAPACITY);
-        a.vcnt[a.e_of_c ? a.e_of_c[i] : i] = vc < a.vcap ? vc : a.vcap;
+        a.vcnt[row_i] = vc < a.vcap ? vc : a.vcap;
         const int64_t p = a.perm[i];
         a.vref[p] = a.x[p];
         if (DIM >= 2) a.vref[a.n + p] = a.y[p];

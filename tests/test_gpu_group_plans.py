@@ -9,7 +9,7 @@ import pytest
 import synth
 
 torch = pytest.importorskip("torch")
-from test_gpu_pair_groups import _check, _gas, _lattice  # noqa: E402
+from test_gpu_pair_groups import SHAPES, _check, _check_step, _gas, _lattice  # noqa: E402
 
 pytestmark = pytest.mark.gpu
 
@@ -83,3 +83,18 @@ def test_more_scan_tiles_than_blocks():
     at = [(a, b, c) for a in far for b in far for c in far]
     pos = np.concatenate([base + np.array(o)[:, None] for o in at], axis=1)
     _check(_gas(pos), "fp64", 1e-10)
+
+
+def _hundred_a_cell():
+    """Two larger particles far off make cells of about a hundred: several groups of 32 home particles."""
+    p = np.concatenate([_lattice((13, 12, 11)), [[60.0, 75.0], [0.0, 0.0], [0.0, 0.0]]], axis=1)
+    return _gas(p, np.concatenate([np.ones(p.shape[1] - 2), [1.6, 1.6]]))
+
+
+LISTED = {**{k: v for k, v in SHAPES.items() if k != "crowded"}, "hundred": _hundred_a_cell}
+
+
+@pytest.mark.parametrize("name", list(LISTED))
+def test_list_build_shapes(name):
+    """Lists of few, of sparse and of many candidates a group against the oracle's pairs and steps."""
+    _check_step(LISTED[name](), 0.15)
