@@ -351,7 +351,7 @@ def run_gpu(args, rank: int, world: int, local_rank: int):
                         "pair_ms_per_launch": pair_ms_avg, "pair_share": pair_ms / ms,
                         "issue_active": None if traffic is None else pair_profile_value(args, "issue_active_frac"),
                         "issue_note": "fraction of the kernel's issue slots used (ncu, the committed summary): "
-                                      "the kernel is issue-bound, the FP32 fraction counts algorithmic flops only"},
+                                      "the kernel is bound by issue and the L1 data pipe, the FP32 fraction counts algorithmic flops only"},
            "graph": None if graph_ms is None else {
                "ms_per_step": graph_ms / args.steps,
                "value": job_value(prob.n, world, args.steps, graph_ms), "list_builds": graph_builds,
@@ -702,10 +702,10 @@ def pair_traffic_bytes(args, profiles_dir: str | None = None):
 
 def kernel_rev() -> str:
     """Identifier of the pair-kernel sources the stored ncu figures belong to
-    (the two pair translation units and the headers they include)."""
+    (the pair and list-build translation units and the headers they include)."""
     import hashlib
     h = hashlib.sha1()
-    for f in ("k_pair.cu", "k_pair_lists.cu", "pair_common.cuh", "step_math.cuh", "csph_internal.cuh"):
+    for f in ("k_pair.cu", "k_pair_lists.cu", "k_list_build.cu", "pair_common.cuh", "step_math.cuh", "csph_internal.cuh"):
         h.update(open(os.path.join(ROOT, "paper_1805_05128_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 

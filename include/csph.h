@@ -104,8 +104,8 @@ typedef struct sph_params {
   int32_t n_units;    /* K <= SPH_MAX_UNITS */
   int32_t unit_dim;   /* dimension of the decomposition: 1, 2 or 3 (<= dim) */
   int32_t n_upd;      /* sph_step rebalances every n_upd steps (0 = never) */
-  int32_t pair_blocks_per_sm; /* resident CTAs per SM of the persistent pair kernel (128 threads,
-                                 one warp per home cell); 0 or more than fit = as many as fit */
+  int32_t pair_blocks_per_sm; /* resident CTAs per SM of the persistent pair kernels (128 threads,
+                                 a warp per group of slots or home cell); 0 or more than fit = as many as fit */
   double theta;       /* eq. (TotalOffset) */
   double sigma;       /* eq. (BalancingOffsetPlusRot) */
   double gamma_b;     /* gamma of eq. (TotalOffset) */

@@ -425,7 +425,8 @@ inline int grid_for(int64_t n, int threads) { return (int)((n + threads - 1) / t
 // Message reported by sph_last_error(NULL) (entry points without a handle).
 void set_global_error(const std::string& msg);
 
-// Launchers (defined in k_step.cu, k_pair.cu, k_vd3.cu).  They enqueue on
+// Launchers (k_step.cu, k_pair.cu, k_pair_lists.cu, k_list_build.cu, k_vd3.cu,
+// k_adjoint.cu).  They enqueue on
 // `st` and return the launch status.
 // d, P, c and the block partials (bounding box, sizes) of a mesh build at the current state
 cudaError_t launch_derive(sph_handle* h, const sph_state& s, cudaStream_t st);

@@ -12,7 +12,7 @@ namespace {
 // Pair evaluation over the Verlet lists: four lanes per slot i (eight slots
 // per warp: the per-slot reductions and set-up are shared by eight slots, and
 // a list of ~90 entries fills its lanes to the last chunk), taken in groups
-// of 32 consecutive slots from a global counter.  The slot's lanes read i's
+// of 8 to 32 consecutive slots (sized at the launch) from a global counter.  The slot's lanes read i's
 // list four entries at a time (particle-major, so the reads are contiguous);
 // each lane decides its entry as k_pair does (FP32 test outside the band of
 // 2^-12 D^c^2, FP64 in the oracle's operation order inside it) and, if the
@@ -26,6 +26,13 @@ namespace {
 // relative to the cells of the build and each pair's shift comes from its
 // neighbour-cell code, so the momentum fluxes stay antisymmetric bit for bit; every
 // order is fixed, so results are reproducible bit for bit.
+//
+// Bound, mixed: the L1 data pipe (86 % of its cycles) and issue (76 %) together:
+// an operand gather touches ~13 line quarters per 32 entries.  A neighbour's
+// position and velocity operands are one 32-byte record read by one load (660 ->
+// 636 us at 1.125M against two arrays).  FP64: the FP64 pipe; the FP32 test runs
+// first over a segment of entries, the accepted ones are compacted and their
+// fluxes evaluated with full lanes (65k ejecta cloud, two steps, 2453 -> 1694 us).
 
 // Lanes per slot of k_pair_lists (a divisor of 32): measured on the 1.125M
 // plate impact, 16 / 8 / 4 / 2 lanes per slot take 0.89 / 0.81 / 0.75 / 0.76 ms.
@@ -88,7 +95,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int half = lane / kSlotLanes, hl = lane % kSlotLanes;   // the slot's group of lanes, lane in it
-  // Work partition.  SPH_SCHED_GLOBAL: groups of 32 consecutive slots from one
+  // Work partition.  SPH_SCHED_GLOBAL: groups of 8 to 32 consecutive slots from one
   // global counter, the last ones of 8 (launch_lists_one).  Units: each unit owns a contiguous range of evaluation
   // slots and a counter; CTA b starts on unit b K / gridDim.x (the CTAs are
   // spread evenly over the units), takes groups of 32 slots of that unit and,

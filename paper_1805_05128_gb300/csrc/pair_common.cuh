@@ -39,7 +39,7 @@ struct PairArgs {
   int adj_words;  // 32-bit words per row
   unsigned long long* counters;
   int* status;
-  unsigned long long* work_counter;   // next cell for the persistent warps (zeroed per launch)
+  unsigned long long* work_counter;   // next group (or home cell) for the persistent warps; zeroed by k_pack
   int group;                           // k_pair: slots per warp and group (at most 32)
   int big;                             // k_pair_lists: slots of a big group (at most 32)
   int64_t big_groups;                  // big groups; the slots after them go out in groups of 8
@@ -54,7 +54,7 @@ struct PairArgs {
   double eta_half, kappa;
   int kernel;
   // reverse mode (k_pair<..., VJP = true>): adjoint operands in slot order,
-  // G = ((dL/da)/m, (dL/ddE)/m), GR2 = (dL/ddrho, rho), and the 11 own-side
+  // G = ((dL/da)/m, (dL/ddE)/m), GR2 = (dL/ddrho, rho) (FP64: its product in y), and the 11 own-side
   // derivatives per particle (particle order) it writes
   const void* G;
   const void* GR2;

@@ -21,7 +21,7 @@ class Tuning:
     """Knobs of a handle that change speed but not the method:
     cell_beta   -- beta of eq. (Dcell): cells (1 + beta) times the minimum size;
     pair_blocks -- resident CTAs per SM of the persistent pair kernel
-                   (4 warps each, one warp per home cell at a time)."""
+                   (4 warps each, one warp per group of slots at a time)."""
     cell_beta: float = 0.0
     pair_blocks: int = 0
     timings: dict = field(default_factory=dict)   # (cell_beta, pair_blocks) -> ms per step
