@@ -522,7 +522,7 @@ def run_extras(args, dev) -> dict:
         "workload": "256 plate impacts, N log-uniform 5k-200k (seed 2018), v U[0.5,2] km/s, gamma U[1.5,3]",
         "particles": n_tot, "steps": 100,
         "batched": {"value": n_tot * 100 / (ms_b * 1e-3), "unit": UNIT, "ms": ms_b,
-                    "form": "one handle, 256 instances, 100 steps in one CUDA graph replay (about 16 kernel "
+                    "form": "one handle, 256 instances, 100 steps in one CUDA graph replay (about 12 kernel "
                             "launches per step inside the graph, not one persistent kernel)", "status": st_b},
         "sequential": {"value": n_tot * 100 / (ms_s * 1e-3), "unit": UNIT, "ms": ms_s,
                        "form": "256 handles, each stepped 100 times eagerly in turn", "status": st_s},
