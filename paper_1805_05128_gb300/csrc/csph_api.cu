@@ -44,7 +44,9 @@ class Workspace {
   void upload(T** p, const std::vector<T>& v) { add(p, sizeof(T) * v.size(), 0, v.data()); }
 
   // Allocates into *base and sets every requested pointer; the copy and the
-  // memset are enqueued on st.
+  // memset are enqueued on st.  A copy from pageable memory may read it after
+  // the call has returned (a host whose memory the device addresses itself), so
+  // an object with uploads lives until the stream has been waited for.
   cudaError_t commit(void** base, cudaStream_t st) {
     size_t end[3], at = 0;
     for (int kind = 0; kind < 3; ++kind) {
@@ -59,14 +61,14 @@ class Workspace {
     cudaError_t e = cudaMalloc(base, at > 0 ? at : 256);
     if (e != cudaSuccess) { *base = nullptr; return e; }
     char* b = static_cast<char*>(*base);
-    std::vector<char> host(end[0]);
+    host_.assign(end[0], 0);
     for (const Item& it : items_) {
       *it.ptr = b + it.at;
-      if (it.kind == 0 && !it.data.empty()) std::memcpy(host.data() + it.at, it.data.data(), it.bytes);
+      if (it.kind == 0 && !it.data.empty()) std::memcpy(host_.data() + it.at, it.data.data(), it.bytes);
     }
-    if (end[0] > 0 && (e = cudaMemcpyAsync(b, host.data(), end[0], cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
+    if (end[0] > 0 && (e = cudaMemcpyAsync(b, host_.data(), end[0], cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
     if (end[1] > end[0] && (e = cudaMemsetAsync(b + end[0], 0, end[1] - end[0], st)) != cudaSuccess) return e;
-    return cudaSuccess;   // (a copy from pageable memory has left `host` when it returns)
+    return cudaSuccess;
   }
 
  private:
@@ -77,6 +79,7 @@ class Workspace {
     std::vector<char> data;
   };
   std::vector<Item> items_;
+  std::vector<char> host_;   // source of the upload
 
   template <typename T>
   void add(T** p, size_t bytes, int kind, const void* data) {
@@ -231,6 +234,7 @@ int sph_init(sph_handle** out, const sph_params* p, int n_instances, const int64
   cudaStream_t st = (cudaStream_t)stream;
   auto bail = [&](int code) {
     g_init_error = h->err;
+    cudaStreamSynchronize(st);   // an upload in flight reads the workspace object
     free_all(h);
     delete h;
     return code;
