@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -373,30 +374,39 @@ __device__ __forceinline__ bool cluster_sum(double (&v)[NV]) {
   return mine;
 }
 
-// CTAs in a cluster for work on n elements, one per `each` of them: up to the 16
-// that fit a cluster here (8 where only the portable size does).  (A sum is
-// bound by the FP64 pipe of the cluster's SMs.)
-template <typename K>
-int cluster_size_for(K kernel, int threads, int64_t n, int64_t each) {
-  static int most = 0;
-  if (most == 0) {
-    int m = 8;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(16);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int active = 0;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) == cudaSuccess && active > 0)
-      m = 16;
-    cudaGetLastError();   // a refused query only means the portable size
-    most = m;
-  }
+// The largest cluster of `kernel` on the current device: 16 CTAs, the largest
+// that exists here, or the portable 8 where 16 are refused.  More than 8 need a
+// function attribute, which belongs to the device it is set on, so the answer is
+// kept per kernel and device (a device past the table is asked each time).
+template <auto kernel>
+int largest_cluster(int threads) {
+  constexpr int kDevices = 64;
+  static std::atomic<int> kept[kDevices];                  // 0: not asked yet
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) { cudaGetLastError(); return 8; }
+  if (dev < kDevices)
+    if (const int m = kept[dev].load(std::memory_order_acquire)) return m;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 16;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int active = 0, m = 8;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&active, kernel, &cfg) == cudaSuccess && active > 0)
+    m = 16;
+  cudaGetLastError();   // a refused query only means the portable size
+  if (dev < kDevices) kept[dev].store(m, std::memory_order_release);
+  return m;
+}
+
+// CTAs in a cluster for work on n elements, one per `each` of them, a power of
+// two up to `most`.  (A sum is bound by the FP64 pipe of the cluster's SMs.)
+inline int cluster_size_for(int most, int64_t n, int64_t each) {
   int c = 1;
   while (c < most && n > each * c) c *= 2;
   return c;

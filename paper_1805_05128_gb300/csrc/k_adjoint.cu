@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(kSumBlock) k_sum_params(int64_t n, const doubl
 }
 
 cudaError_t launch_sum_params(int64_t n, const double* par, double* out, cudaStream_t st) {
-  return launch_clusters(k_sum_params, 1, cluster_size_for(k_sum_params, kSumBlock, n, 4096), kSumBlock, st, n, par, out);
+  const int per = cluster_size_for(largest_cluster<k_sum_params>(kSumBlock), n, 4096);
+  return launch_clusters(k_sum_params, 1, per, kSumBlock, st, n, par, out);
 }
 
 }  // namespace

@@ -1142,7 +1142,7 @@ cudaError_t launch_exclusive_scan(int32_t* cnt, const int64_t* total, int32_t* s
 // (launch_exclusive_scan's two kernels are counted by its callers)
 
 cudaError_t launch_conservation(sph_handle* h, const sph_state& s, double* out, cudaStream_t st) {
-  const int per = cluster_size_for(k_conservation, kSumBlock, h->n / h->n_inst, 4096);
+  const int per = cluster_size_for(largest_cluster<k_conservation>(kSumBlock), h->n / h->n_inst, 4096);
   CKL(launch_clusters(k_conservation, h->n_inst, per, kSumBlock, st, s, h->inst_off, out));
   h->launches += 1;
   return cudaGetLastError();

@@ -1,4 +1,5 @@
 """Host code of the library against a stand-in runtime (tests/host_runtime.py)."""
+import ctypes as C
 import shutil
 
 import pytest
@@ -26,3 +27,26 @@ def scenario_upload(so, precision, beta):
 @pytest.mark.parametrize("beta", [0, 1])
 def test_uploads_outlive_their_copies(so, precision, beta):
     assert host_runtime.run(so, "test_host_runtime:scenario_upload", precision, beta) == "(True, 0)"
+
+
+def scenario_devices(so):
+    """The totals and the parameter adjoints on a device that is not the first one used: launch errors, clusters."""
+    H = host_runtime.Host(so)
+    n, got = 70000, []
+    for dev in (0, 1, 70, 71, 0):
+        H.L.fake_set_device(dev)
+        s = H.state(n)
+        h = H.handle(s)
+        out = H.array(5)
+        H.launches()
+        rc = [H.L.sph_conservation(h, C.byref(s), out.ctypes.data, None)]
+        ck = H.abi.sph_ckpt(state=s, dt=H.array(1).ctypes.data)
+        adj = H.state(n)
+        rc.append(H.L.sph_step_adjoint(h, C.byref(ck), 1, C.byref(adj), C.byref(adj), H.array(2).ctypes.data, None))
+        got.append(rc + [c for name, blocks, c in H.launches() if c > 1])
+        H.abi.sph_destroy(h)
+    return got
+
+
+def test_clusters_on_every_device(so):
+    assert host_runtime.run(so, "test_host_runtime:scenario_devices") == str([[0, 0, 16, 16]] * 5)
