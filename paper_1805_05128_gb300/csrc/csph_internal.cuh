@@ -430,6 +430,23 @@ cudaError_t launch_clusters(void (*kernel)(KArgs...), int clusters, int per, int
 // --------------------------------------------------------------------------
 // Host helpers shared by the translation units
 // --------------------------------------------------------------------------
+// The SMs of the device and the resident blocks of `kernel` on each, asked once.
+// Both are kept in one word, so that a thread sees both or neither.
+struct Resident { int sms, per_sm; };
+template <auto kernel>
+Resident resident_blocks(int threads) {
+  static std::atomic<uint64_t> kept{0};                    // 0: not asked yet
+  const uint64_t k = kept.load(std::memory_order_relaxed);
+  if (k) return {(int)(k >> 32), (int)(uint32_t)k};
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, 0);
+  if (per_sm < 1) per_sm = 1;
+  if (sms > 0) kept.store((uint64_t)(uint32_t)sms << 32 | (uint32_t)per_sm, std::memory_order_relaxed);
+  return {sms, per_sm};
+}
+
 inline int grid_for(int64_t n, int threads) { return (int)((n + threads - 1) / threads); }
 
 // Message reported by sph_last_error(NULL) (entry points without a handle).

@@ -261,14 +261,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairAr
 
 template <bool MIXED, int DIM>
 cudaError_t launch_one(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
-  static int sms = 0, per_sm = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_list_build<MIXED, DIM>, kPairBlock, 0);
-    if (per_sm < 1) per_sm = 1;
-  }
+  const auto [sms, per_sm] = resident_blocks<k_list_build<MIXED, DIM>>(kPairBlock);
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
   return launch_chained(k_list_build<MIXED, DIM>, dim3(sms * b), dim3(kPairBlock), st, args);
 }

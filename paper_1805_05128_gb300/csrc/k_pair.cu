@@ -637,14 +637,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
 // pair_blocks_per_sm (0 = as many as fit) and by the number of groups.
 template <bool MIXED, int DIM, int MODE, int G, bool HLL, bool EXTRA>
 cudaError_t launch_lanes(const PairArgs& args, int blocks_per_sm, cudaStream_t st) {
-  static int sms = 0, per_sm = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair<MIXED, DIM, MODE, G, HLL, EXTRA>, kPairBlock, 0);
-    if (per_sm < 1) per_sm = 1;
-  }
+  const auto [sms, per_sm] = resident_blocks<k_pair<MIXED, DIM, MODE, G, HLL, EXTRA>>(kPairBlock);
   PairArgs a = args;
   a.group = 32 / G;
   // a group of fewer slots while not every SM has four warps at work

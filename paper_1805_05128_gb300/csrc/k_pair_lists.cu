@@ -509,15 +509,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
 
 template <bool MIXED, int DIM, bool HLL, bool EXTRA, bool STAGE, int KERN>
 cudaError_t launch_lists_one(const PairArgs& args_in, int blocks_per_sm, cudaStream_t st) {
-  static int sms = 0, per_sm = 0;
-  if (sms == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_pair_lists<MIXED, DIM, HLL, EXTRA, STAGE, KERN>,
-                                                  kPairBlock, 0);
-    if (per_sm < 1) per_sm = 1;
-  }
+  const auto [sms, per_sm] = resident_blocks<k_pair_lists<MIXED, DIM, HLL, EXTRA, STAGE, KERN>>(kPairBlock);
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
   int grid = sms * b;
   // Groups of 32 slots share the set-up and the FP64 rate formation best (a

@@ -1,6 +1,8 @@
 """Host code of the library against a stand-in runtime (tests/host_runtime.py)."""
 import ctypes as C
 import shutil
+import threading
+import time
 
 import pytest
 
@@ -50,3 +52,35 @@ def scenario_devices(so):
 
 def test_clusters_on_every_device(so):
     assert host_runtime.run(so, "test_host_runtime:scenario_devices") == str([[0, 0, 16, 16]] * 5)
+
+
+def scenario_first_use(so, beta):
+    """Two threads that need a kernel's grid for the first time at once: both launch, the same blocks."""
+    H = host_runtime.Host(so)
+    s = H.state(50000)
+    hs = [H.handle(s, cell_beta=0.15 * beta) for _ in range(2)]
+    for h in hs:
+        H.L.sph_hold_rates(h)
+    H.launches()
+    H.L.fake_query_ms(400)          # the occupancy query takes this long
+    rc = [None, None]
+
+    def step(k):
+        rc[k] = H.L.sph_step(hs[k], C.byref(s), 1, None, None)
+
+    threads = [threading.Thread(target=step, args=(k,)) for k in (0, 1)]
+    threads[0].start()
+    time.sleep(0.1)
+    threads[1].start()
+    for t in threads:
+        t.join()
+    grids = {}
+    for name, blocks, _ in H.launches():
+        if "k_pair" in name or "k_list_build" in name:
+            grids.setdefault(name, []).append(blocks)
+    return rc, sorted(len(g) for g in grids.values()), all(len(set(g)) == 1 for g in grids.values())
+
+
+@pytest.mark.parametrize("beta", [0, 1])
+def test_first_use_by_two_threads(so, beta):
+    assert host_runtime.run(so, "test_host_runtime:scenario_first_use", beta) == str(([0, 0], [2] * (1 + beta), True))
