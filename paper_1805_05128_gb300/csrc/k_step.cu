@@ -1039,7 +1039,7 @@ cudaError_t launch_build_grid(sph_handle* h, const sph_state& s, cudaStream_t st
   CKL(launch_chained(k_scan_down, dim3(tiles), dim3(kBlock), st, h->cell_count, h->total_cells, h->scan_sums, h->cell_start, h->n, gate));
   CKL(launch_chained(k_cell_scatter, dim3(capped_grid(grid_for(h->n, kBlock))), dim3(kBlock), st, a));
   CKL(launch_chained(k_cell_sort, dim3(capped_grid(grid_for(h->cell_cap * 32, kBlock))), dim3(kBlock), st, a));
-  h->launches += 5;
+  h->launches += 6;
   // a mesh built outside the Verlet sequence changes the slot order under the lists
   if (!gate && h->verlet) return cudaMemsetAsync(&h->vflag[1], 0xff, sizeof(int), st);
   return cudaGetLastError();

@@ -4,6 +4,7 @@ import shutil
 import threading
 import time
 
+import numpy as np
 import pytest
 
 import host_runtime
@@ -84,3 +85,49 @@ def scenario_first_use(so, beta):
 @pytest.mark.parametrize("beta", [0, 1])
 def test_first_use_by_two_threads(so, beta):
     assert host_runtime.run(so, "test_host_runtime:scenario_first_use", beta) == str(([0, 0], [2] * (1 + beta), True))
+
+
+def scenario_counter(so):
+    """The calls whose count of kernel launches (sph_profile_read) is not the number of launches made."""
+    H = host_runtime.Host(so)
+    abi, L, n = H.abi, H.L, 5000
+    out, gen, dts = H.array(6 * n), H.array(3 * 8), H.array(16)
+    ints = H.array(2 * n, np.int32)
+    bp, cnt = abi.sph_balance_params(), C.c_int64()
+    units = dict(n_units=8, unit_dim=3, n_upd=2, generators=gen.ctypes.data)
+    handles = {"search": {}, "fp64": dict(precision=0), "lists": dict(cell_beta=0.15), "order2": dict(order=2),
+               "units": units, "units lists": dict(units, cell_beta=0.15),
+               "units sched": dict(units, cell_beta=0.15, unit_sched=1), "batched": dict(offsets=[0, 700, n]),
+               "batched lists": dict(offsets=[0, 700, n], cell_beta=0.15)}
+    wrong = []
+    for name, kw in handles.items():
+        s, adj = H.state(n), H.state(n)
+        h = H.handle(s, **kw)
+        ck = abi.sph_ckpt(state=s, dt=dts.ctypes.data, rates_from_state=1)
+        ck64 = abi.sph_ckpt(state=s, dt=dts.ctypes.data, reverse_fp64=1)
+        S, o = C.byref(s), out.ctypes.data
+        calls = {"eval": lambda: L.sph_eval_rates(h, S, None), "step": lambda: L.sph_step(h, S, 1, None, None),
+                 "3 steps": lambda: L.sph_step(h, S, 3, o, None), "2 given steps": lambda: L.sph_step_dt(h, S, 2, dts.ctypes.data, o, None),
+                 "build": lambda: L.sph_build_cells(h, S, None), "cfl": lambda: L.sph_cfl_dt(h, S, o, None),
+                 "totals": lambda: L.sph_conservation(h, S, o, None), "cells": lambda: L.sph_cell_index(h, S, ints.ctypes.data, None, None),
+                 "pairs": lambda: L.sph_pair_list(h, S, n, ints.ctypes.data, ints.ctypes.data, C.byref(cnt), None)}
+        if name in ("search", "fp64", "lists"):
+            calls["adjoint"] = lambda: L.sph_step_adjoint(h, C.byref(ck), 3, C.byref(adj), C.byref(adj), o, None)
+            calls["adjoint fp64"] = lambda: L.sph_step_adjoint(h, C.byref(ck64), 3, C.byref(adj), C.byref(adj), o, None)
+        if "units" in name:
+            calls["assign"] = lambda: L.voronoi_assign(h, S, gen.ctypes.data, 8, 3, ints.ctypes.data, None, None)
+            calls["balance"] = lambda: L.voronoi_balance(h, S, gen.ctypes.data, 8, 3, None, C.byref(bp), None, None)
+        for call, f in calls.items():
+            L.sph_profile(h, 0)
+            H.launches()
+            rc, counted = f(), C.c_int64()
+            made = len(H.launches())
+            L.sph_profile_read(h, None, None, C.byref(counted))
+            if rc != 0 or counted.value != made or made == 0:
+                wrong.append((name, call, rc, counted.value, made))
+        abi.sph_destroy(h)
+    return wrong
+
+
+def test_launch_counter(so):
+    assert host_runtime.run(so, "test_host_runtime:scenario_counter") == "[]"
