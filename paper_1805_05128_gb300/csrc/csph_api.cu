@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -58,10 +59,10 @@ class Workspace {
       end[kind] = at;
     }
     *base = nullptr;
+    host_.assign(end[0], 0);
     cudaError_t e = cudaMalloc(base, at > 0 ? at : 256);
     if (e != cudaSuccess) { *base = nullptr; return e; }
     char* b = static_cast<char*>(*base);
-    host_.assign(end[0], 0);
     for (const Item& it : items_) {
       *it.ptr = b + it.at;
       if (it.kind == 0 && !it.data.empty()) std::memcpy(host_.data() + it.at, it.data.data(), it.bytes);
@@ -88,6 +89,22 @@ class Workspace {
     items_.push_back(std::move(it));
   }
 };
+
+// One more block of workspace for the handle: request(ws) names the arrays.  Where
+// an allocation fails, on the host or the device, no pointer is set.
+template <typename F>
+cudaError_t add_workspace(sph_handle* h, cudaStream_t st, F&& request) {
+  try {
+    Workspace ws;
+    request(ws);
+    h->blocks.push_back(nullptr);
+    const cudaError_t e = ws.commit(&h->blocks.back(), st);
+    if (!h->blocks.back()) h->blocks.pop_back();
+    return e;
+  } catch (const std::bad_alloc&) {
+    return cudaErrorMemoryAllocation;
+  }
+}
 
 void free_all(sph_handle* h) {
   for (void* p : h->blocks)
@@ -746,14 +763,6 @@ namespace {
 constexpr int kAdjStored = 13;
 constexpr int kAdjW = 16;
 
-// One more block of workspace for the handle.  Where the allocation fails, no pointer is set.
-cudaError_t commit(sph_handle* h, Workspace& ws, cudaStream_t st) {
-  void* base = nullptr;
-  const cudaError_t e = ws.commit(&base, st);
-  if (base) h->blocks.push_back(base);
-  return e;
-}
-
 sph_state adj_work_state(sph_handle* h, const sph_state& ck) {
   const int64_t n = h->n;
   double* w = h->adj_W;
@@ -814,23 +823,25 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
   h->last_stream = st;
   const int64_t n = h->n;
   if (!h->adj_G) {
-    Workspace ws;
-    ws.raw(&h->adj_G, n);
-    ws.raw(&h->adj_GR, n);
-    ws.raw(&h->adj_pair, (size_t)11 * n);
-    ws.raw(&h->adj_par, (size_t)2 * n);
-    ws.zeroed(&h->adj_W, (size_t)kAdjW * n);
-    CK(h, commit(h, ws, st));
+    auto arrays = [&](Workspace& ws) {
+      ws.raw(&h->adj_G, n);
+      ws.raw(&h->adj_GR, n);
+      ws.raw(&h->adj_pair, (size_t)11 * n);
+      ws.raw(&h->adj_par, (size_t)2 * n);
+      ws.zeroed(&h->adj_W, (size_t)kAdjW * n);
+    };
+    CK(h, add_workspace(h, st, arrays));
   }
   // FP64 pair derivatives on a mixed-precision handle (the forward replay stays mixed)
   const bool rev64 = h->dp.precision == SPH_PREC_MIXED && ck->reverse_fp64 != 0;
   if (rev64 && !h->adj64_A) {
-    Workspace ws;
-    ws.raw(reinterpret_cast<D4**>(&h->adj64_A), n);
-    ws.raw(reinterpret_cast<D4**>(&h->adj64_B), n);
-    ws.raw(reinterpret_cast<D2**>(&h->adj64_C), n);
-    ws.raw(&h->adj64_rho, n);
-    CK(h, commit(h, ws, st));
+    auto arrays = [&](Workspace& ws) {
+      ws.raw(reinterpret_cast<D4**>(&h->adj64_A), n);
+      ws.raw(reinterpret_cast<D4**>(&h->adj64_B), n);
+      ws.raw(reinterpret_cast<D2**>(&h->adj64_C), n);
+      ws.raw(&h->adj64_rho, n);
+    };
+    CK(h, add_workspace(h, st, arrays));
   }
   if (n_steps > h->adj_store_steps) {
     if (h->adj_store) {
@@ -840,9 +851,8 @@ int sph_step_adjoint(sph_handle* h, const sph_ckpt* ck, int n_steps, const sph_s
     }
     h->adj_store = nullptr;
     h->adj_store_steps = 0;
-    Workspace ws;
-    ws.raw(&h->adj_store, (size_t)n_steps * kAdjStored * n);
-    CK(h, commit(h, ws, st));
+    auto arrays = [&](Workspace& ws) { ws.raw(&h->adj_store, (size_t)n_steps * kAdjStored * n); };
+    CK(h, add_workspace(h, st, arrays));
     h->adj_store_steps = n_steps;
   }
   sph_state W = adj_work_state(h, ck->state);

@@ -131,3 +131,29 @@ def scenario_counter(so):
 
 def test_launch_counter(so):
     assert host_runtime.run(so, "test_host_runtime:scenario_counter") == "[]"
+
+
+def scenario_host_memory(so, reverse_fp64):
+    """sph_step_adjoint with the k-th host allocation refused, k = 0, 1, ...: an error code each time, then success."""
+    H = host_runtime.Host(so)
+    s, adj = H.state(3000), H.state(3000)
+    ck = H.abi.sph_ckpt(state=s, dt=H.array(3).ctypes.data, reverse_fp64=reverse_fp64)
+    par, codes = H.array(2), []
+    for k in range(200):
+        h = H.handle(s)
+        H.launches()
+        H.L.fake_fail_new(k)
+        codes.append(H.L.sph_step_adjoint(h, C.byref(ck), 3, C.byref(adj), C.byref(adj), par.ctypes.data, None))
+        H.L.fake_fail_new(-1)
+        again = H.L.sph_step_adjoint(h, C.byref(ck), 3, C.byref(adj), C.byref(adj), par.ctypes.data, None)
+        H.abi.sph_destroy(h)
+        if again != 0:
+            return k, again
+        if codes[-1] == 0:
+            break
+    return len(codes) > 3, set(codes[:-1]) == {H.abi.SPH_ERR_CUDA}, codes[-1]
+
+
+@pytest.mark.parametrize("reverse_fp64", [0, 1])
+def test_no_exception_leaves_the_adjoint(so, reverse_fp64):
+    assert host_runtime.run(so, "test_host_runtime:scenario_host_memory", reverse_fp64) == "(True, True, 0)"
