@@ -15,8 +15,14 @@
 //
 // The test runs in FP32 in both precisions (mixed handles on the packed
 // offsets from the cell origins, FP64 handles on offsets from the cell's first
-// particle scaled to a cell edge of ~1) and accepts r^2 - R^2 < 2^-12 D^c^2, a
-// superset of the radius: k_pair_lists decides each entry exactly.
+// particle scaled to a cell edge of ~1).  Mixed handles accept r^2 - R^2 < 2^-12
+// D^c^2, a superset of the radius: k_pair_lists decides each entry exactly.  FP64
+// handles decide the candidates within 2^-17 D^c^2 of R^2 in FP64, so that a row
+// holds the radius and nothing beyond it, however far the particle sizes lie
+// apart.  (Their FP32 error is below 2^-19 D^c^2: offsets of at most two edges,
+// rounded to 2^-23 D^c each, three products of at most D^c^2, and an R of four
+// roundings; a superset like the mixed one would hold ten times the radius
+// between particles 600 times smaller than the largest.)
 // Bound by issue (77 % of the slots) and the latency of its short phases:
 // 659 us at 1.125M particles, 768 us at 1M droplet particles.  Rows gathered in
 // shared memory, one append per test and lane, and flushed at the end (33 KB a
@@ -39,6 +45,24 @@ __device__ __forceinline__ float warp_max(float v) {
   float r;
   asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
   return r;
+}
+
+// The candidates of `mask` (places in `slots`) that lie within R of slot i, in
+// FP64 and the oracle's operation order.  A call, because it is rare and its
+// code inside the drain cost the whole build 3 %: two steps of the 65k ejecta
+// cloud 1657 us without the decision, 1680 inlined, 1656 called.
+template <int DIM>
+__device__ __noinline__ unsigned decide_exactly(const D4* A, int i, unsigned mask, const int32_t* slots, double kh) {
+  unsigned left = mask;
+  for (unsigned m = mask; m; m &= m - 1) {
+    const int c = __ffs(m) - 1;
+    const D4 Ai = A[i], Aj = A[slots[c]];
+    const double r2 = Pair<false, DIM>::r2_of(__dsub_rn(Aj.x, Ai.x), DIM >= 2 ? __dsub_rn(Aj.y, Ai.y) : 0.0,
+                                              DIM >= 3 ? __dsub_rn(Aj.z, Ai.z) : 0.0);
+    const double R = __dmul_rn(kh, __dadd_rn(Ai.w, Aj.w));
+    if (!(r2 < __dmul_rn(R, R))) left &= ~(1u << c);
+  }
+  return left;
 }
 
 // Resident blocks: mixed 8 / 7 / 6 took 5305 / 5212 / 5230 us for five steps of
@@ -97,7 +121,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairAr
       const V4 O = A[hs];
       fx = O.x; fy = O.y; fz = O.z;
     }
-    const float band = 0x1p-12f * dct * dct;
+    const float band = (MIXED ? 0x1p-12f : 0x1p-17f) * dct * dct;
     auto frame = [&](const V4& R, int ox, int oy, int oz) {
       float4 S;
       if constexpr (MIXED) {
@@ -142,6 +166,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairAr
         const float2 kh2 = make_float2(a.kh_f, a.kh_f), kd2 = make_float2(khdi, khdi);
         const float2 nk2 = make_float2(-a.kh_f, -a.kh_f), nd2 = make_float2(-khdi, -khdi);
         unsigned mask = 0;
+        float near = __int_as_float(0x7f800000);             // the least |r^2 - R^2| (FP64 handles)
 #pragma unroll
         for (int c = 0; c < 32; c += 4) {
           if (c >= nc) break;
@@ -166,6 +191,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairAr
             const float2 diff = fma2(fma2(nk2, d, nd2), fma2(kh2, d, kd2), r2);   // r^2 - R^2
             if (diff.x < band) mask |= 1u << (c + 2 * k);
             if (diff.y < band) mask |= 2u << (c + 2 * k);
+            if constexpr (!MIXED) near = fminf(near, fminf(fabsf(diff.x), fabsf(diff.y)));
           }
         }
         if (nc < 32) mask &= (1u << nc) - 1u;
@@ -179,6 +205,10 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 6) k_list_build(PairAr
           const int first = __ffs(own) - 1;
           const unsigned k = (unsigned)(i - __shfl_sync(0xffffffffu, jc, first));
           if (k < (unsigned)__popc(own)) mask &= ~(1u << (first + k));
+        }
+        if constexpr (!MIXED) {
+          // too close to call in FP32, which is rare: the lane decides its candidates in FP64
+          if (near <= band) mask = decide_exactly<DIM>(A, i, mask, &qslot[warp][at], a.kh);
         }
         for (int h8 = 0; h8 < nh; h8 += 8) {   // (the masks of lanes past nh are empty)
 #pragma unroll
