@@ -406,7 +406,7 @@ int largest_cluster(int threads) {
 
 // CTAs in a cluster for work on n elements, one per `each` of them, a power of
 // two up to `most`.  (A sum is bound by the FP64 pipe of the cluster's SMs.)
-inline int cluster_size_for(int most, int64_t n, int64_t each) {
+__host__ __device__ inline int cluster_size_for(int most, int64_t n, int64_t each) {
   int c = 1;
   while (c < most && n > each * c) c *= 2;
   return c;

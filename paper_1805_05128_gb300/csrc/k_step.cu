@@ -6,6 +6,7 @@
 // Every per-particle kernel runs on "segmented" blocks: block b covers the
 // particles [blk_start[b], blk_end[b]) of one instance, so per-instance
 // reductions are fixed-order reductions over whole blocks (no atomics).
+#include <algorithm>
 #include <cfloat>
 #include <climits>
 
@@ -920,19 +921,24 @@ __global__ void k_scatter_back(int64_t n, PermArrays a, const char* scratch, int
 
 // ---------------------------------------------------------------------------
 // FP64 conservation sums per instance, fixed order: one cluster of CTAs per
-// instance, its threads striding over the instance's particles.  A single CTA
-// per instance (one SM's FP64 pipe, two loads in flight) took 3.3 ms on 1M
-// particles, a cluster of 16 takes 0.1 ms.
+// instance, its threads striding over the instance's particles.  The CTAs that
+// take part follow from the instance's own size, not from the launch's clusters
+// (those past them add zeros), so that an instance's totals are the same bits
+// whatever shares its handle.  A single CTA per instance (one SM's FP64 pipe,
+// two loads in flight) took 3.3 ms on 1M particles, a cluster of 16 takes 0.1 ms.
 // ---------------------------------------------------------------------------
+constexpr int64_t kSumEach = 4096;   // particles per CTA of a sum
 __global__ void __launch_bounds__(kSumBlock) k_conservation(sph_state s, const int64_t* __restrict__ inst_off, double* out) {
   namespace cg = cooperative_groups;
   const cg::cluster_group cl = cg::this_cluster();
-  const int per = (int)cl.num_blocks();
+  const int per = (int)cl.num_blocks(), rank = (int)cl.block_rank();
   const int b = blockIdx.x / per;
   double acc[5] = {0, 0, 0, 0, 0};
-  const int64_t p1 = inst_off[b + 1], stride = (int64_t)per * kSumBlock;
+  const int64_t p0 = inst_off[b], p1 = inst_off[b + 1];
+  const int parts = cluster_size_for(per, p1 - p0, kSumEach);   // the largest instance's is per: see the launch
+  const int64_t stride = (int64_t)parts * kSumBlock;
 #pragma unroll 2
-  for (int64_t p = inst_off[b] + (int64_t)cl.block_rank() * kSumBlock + threadIdx.x; p < p1; p += stride) {
+  for (int64_t p = rank < parts ? p0 + (int64_t)rank * kSumBlock + threadIdx.x : p1; p < p1; p += stride) {
     const double m = s.m[p];
     acc[0] += m;
     acc[1] += m * ld(s.vx, p);
@@ -1142,7 +1148,9 @@ cudaError_t launch_exclusive_scan(int32_t* cnt, const int64_t* total, int32_t* s
 // (launch_exclusive_scan's two kernels are counted by its callers)
 
 cudaError_t launch_conservation(sph_handle* h, const sph_state& s, double* out, cudaStream_t st) {
-  const int per = cluster_size_for(largest_cluster<k_conservation>(kSumBlock), h->n / h->n_inst, 4096);
+  int64_t most = 0;                    // the largest instance
+  for (int b = 0; b < h->n_inst; ++b) most = std::max(most, h->inst_off_h[b + 1] - h->inst_off_h[b]);
+  const int per = cluster_size_for(largest_cluster<k_conservation>(kSumBlock), most, kSumEach);
   CKL(launch_clusters(k_conservation, h->n_inst, per, kSumBlock, st, s, h->inst_off, out));
   h->launches += 1;
   return cudaGetLastError();
