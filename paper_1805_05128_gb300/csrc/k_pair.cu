@@ -342,6 +342,7 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
     };
 
     auto flush = [&]() {
+      [[maybe_unused]] const unsigned flushed = nfull;         // entries of the slot that earlier flushes took
       nfull += (unsigned)cnt;
       if constexpr (kOrdered) {
         // The slot's lanes evaluate consecutive entries; then each of them adds
@@ -378,7 +379,9 @@ __global__ void __launch_bounds__(kPairBlock, (MODE == kModeVjp || MODE == kMode
           }
         }
       } else {
-        for (int k = hl; k < cnt; k += G) {
+        // Lane hl takes the slot's entries hl, hl + G, ... counted over its flushes:
+        // when one falls depends on the other slots of the group, the sums do not.
+        for (int k = (int)((unsigned)(hl - (int)flushed) % G); k < cnt; k += G) {
           const unsigned ent = list[warp][home][k];
           // (the two minima change nothing on a finite state; on one with infinite
           // sizes, which is latched, they keep the accesses in bounds)

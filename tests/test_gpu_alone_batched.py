@@ -1,6 +1,7 @@
 """What an instance of a batched handle gets is what it gets alone, bit for
 bit, where the instances sharing the handle could show: the totals of
-instances of any sizes."""
+instances of any sizes, and the FP64 sums of particles with so many
+neighbours that a group's lists are flushed in the middle of its scan."""
 import numpy as np
 import pytest
 
@@ -31,3 +32,27 @@ def test_totals_alone_and_batched(sizes):
         one = Simulation(q, precision="fp64", units=0)
         assert np.array_equal(one.conservation().cpu().numpy()[0], got[b]), sizes[b]
         one.close()
+
+
+@pytest.mark.parametrize("order,solver", [(1, "acoustic"), (1, "hll"), (2, "acoustic")])
+@pytest.mark.parametrize("before", [(1,), (5, 3), (7,) * 9])
+def test_many_neighbours_alone_and_batched(before, order, solver):
+    """Up to 330 neighbours, more than a list holds between two flushes (224)."""
+    from paper_1805_05128_gb300 import Simulation
+    probs = [_gas(_lattice((n, 1, 1), seed=n), seed=n) for n in before] + [_gas(_lattice((11, 9, 8)))]
+    for q in probs:
+        q.eta = 2.15
+    pos = np.stack([probs[-1].arrays[k] for k in "xyz"])
+    d = np.cbrt(probs[-1].arrays["m"] / probs[-1].arrays["rho"])
+    near = np.linalg.norm(pos[:, :, None] - pos[:, None], axis=0) < 2.15 * (d[:, None] + d)
+    assert near.sum(0).max() > 224
+    kw = dict(precision="fp64", units=0, order=order, solver=solver)
+    sim, one = Simulation(probs, cell_cap=1 << 18, **kw), Simulation(probs[-1], **kw)
+    sim.eval_rates()
+    one.eval_rates()
+    g, o, lo = sim.numpy(), one.numpy(), sum(before)
+    assert sim.read_status() == 0
+    for k in ("ax", "ay", "az", "drho", "dE"):
+        assert np.any(o[k]) and np.array_equal(g[k][lo:], o[k]), k
+    sim.close()
+    one.close()
