@@ -65,6 +65,12 @@ __device__ __forceinline__ T slot_sum(const Kahan<T>& k) {
   return v;
 }
 
+// Sum over the warp in 64 bits.
+__device__ __forceinline__ unsigned long long warp_total(unsigned v) {
+  const unsigned hi = __reduce_add_sync(0xffffffffu, v >> 16), lo = __reduce_add_sync(0xffffffffu, v & 0xffffu);
+  return ((unsigned long long)hi << 16) + lo;
+}
+
 template <bool MIXED, int DIM, bool HLL = false, bool EXTRA = true, bool STAGE = false, int KERN = SPH_KERNEL_CUBIC>
 __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairArgs a) {
   chain_entry();
@@ -72,9 +78,11 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
   using T = typename P::T;
   using V4 = typename P::V4;
   using VC = typename P::VC;
-  __shared__ float res[kWarps][6][32];            // per slot of the group: sums of rho, a (3), E, and dmax
+  // Evaluated slots whose rates are still to be formed (pend of them): sums of rho, a (3), E, and dmax
+  __shared__ float res[kWarps][6][32];
   __shared__ double res64[kWarps][6][MIXED ? 1 : 32];
   __shared__ unsigned res_n[kWarps][32];
+  __shared__ int res_i[kWarps][32];              // the slots
   __shared__ long long t_start[kWarps];          // timed loads: start of the warp's slot iteration
   // unit shifts (-1, 0, 1) per axis of each neighbour-cell code; a table read
   // and three multiplies are cheaper than the integer divisions and
@@ -126,7 +134,9 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
     u_cur[warp] = u < a.K ? u : a.K - 1;
     u_left[warp] = a.K;
   }
-  for (;;) {
+  int pend = 0;
+  unsigned tf = 0, tc = 0, te = 0;   // the lane's pairs, entries and exact decisions
+  for (bool more = true; more;) {
     // slots in 32 bits: list entries hold slot indices in 27 bits
     int g0 = 0, g1 = 0;
     if (a.unit_sched == SPH_SCHED_GLOBAL) {
@@ -135,10 +145,12 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       gw = __shfl_sync(0xffffffffu, gw, 0);
       const bool big = (int64_t)gw < a.big_groups;
       const int64_t at = big ? a.big * (int64_t)gw : a.big * a.big_groups + kSlotsPerWarp * ((int64_t)gw - a.big_groups);
-      if (at >= a.n) break;
-      g0 = (int)at;
-      const int64_t end = at + (big ? a.big : kSlotsPerWarp);
-      g1 = end < a.n ? (int)end : (int)a.n;
+      more = at < a.n;
+      if (more) {                                            // else an empty group at slot 0
+        const int64_t end = at + (big ? a.big : kSlotsPerWarp);
+        g0 = (int)at;
+        g1 = end < a.n ? (int)end : (int)a.n;
+      }
     } else {
       int ok = 0;
       if (lane == 0) {
@@ -164,13 +176,12 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
         t_grp[warp] = t;
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) break;
+      more = ok != 0;
       g0 = __shfl_sync(0xffffffffu, g0, 0);
       g1 = __shfl_sync(0xffffffffu, g1, 0);
     }
     int unit_run = -1;
     unsigned unit_load = 0;
-    unsigned tf = 0, tc = 0, te = 0;
     // Half h of the warp takes slots g0 + 2q + h, q = 0..15.  The list reads
     // are software-pipelined: the next chunk of entries (and, across slots,
     // the next slot's first chunk and count) is requested before the current
@@ -379,7 +390,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       }
       if (iv) {
         if (hl == 0) {
-          const int r = i - g0;
+          const int r = pend + i - g0;
           const T vals[6] = {srho, sfx, sfy, sfz, sq, dm};
 #pragma unroll
           for (int qv = 0; qv < 6; ++qv) {
@@ -387,6 +398,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
             else res64[warp][qv][r] = (double)vals[qv];
           }
           res_n[warp][r] = nacc;
+          if (g1 - g0 < 32) res_i[warp][r] = i;
           tf += nacc;
           tc += (unsigned)cnt;
         }
@@ -411,11 +423,19 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       }
     }
     __syncwarp();
-    {
-      const int64_t i = g0 + lane;                     // one slot of the group per lane
+    pend += g1 - g0;
+    // The rates of the pending slots, one per lane, once another group of this size
+    // does not fit (groups never get larger) and at the end; a unit's at once, for
+    // its times.  Formed after every group of 8, their FP64 arithmetic ran with a
+    // quarter of the lanes, which, with the counters' atomics of every group (now
+    // one set per warp), bound short lists: 90k particles of a plane 57 -> 37 us,
+    // 100k of a line 55 -> 30, 300k dilute ones 104 -> 78; long ones of groups of 32
+    // are 0.2 % slower (1.125M: 728 -> 729).
+    if (pend > 0 && (!more || pend + g1 - g0 > 32 || a.unit_sched != SPH_SCHED_GLOBAL)) {
+      const int i = g1 - g0 == 32 ? g0 + lane : (lane < pend ? res_i[warp][lane] : 0);
       long long key = LLONG_MAX;
       int bi = 0;
-      if (i < g1) {
+      if (lane < pend) {
         auto rv = [&](int qv) -> double {
           if constexpr (MIXED) return (double)res[warp][qv][lane];
           else return res64[warp][qv][lane];
@@ -470,32 +490,33 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
       if (a.kick2_cfl) {
         // one atomic per warp when the group lies in one instance (the usual case)
         const int b0 = __shfl_sync(0xffffffffu, bi, 0);
-        if (__all_sync(0xffffffffu, i >= g1 || bi == b0)) {
+        if (__all_sync(0xffffffffu, lane >= pend || bi == b0)) {
 #pragma unroll
           for (int o = 16; o > 0; o >>= 1) {
             const long long q = __shfl_xor_sync(0xffffffffu, key, o);
             key = q < key ? q : key;
           }
           if (lane == 0) atomicMin(&a.dt_key[b0], key);
-        } else if (i < g1) {
+        } else if (lane < pend) {
           atomicMin(&a.dt_key[bi], key);
         }
       }
+      pend = 0;
     }
     __syncwarp();
-    te = __reduce_add_sync(0xffffffffu, te);
-    tf = __reduce_add_sync(0xffffffffu, tf);
-    tc = __reduce_add_sync(0xffffffffu, tc);
-    if (lane == 0) {
-      atomicAdd(&a.counters[0], (unsigned long long)tf);
-      atomicAdd(&a.counters[1], (unsigned long long)tc);
-      atomicAdd(&a.counters[2], (unsigned long long)te);
-      if (a.unit_sched != SPH_SCHED_GLOBAL) {         // the unit's first start and last end
-        unsigned long long t_end;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
-        atomicMin(&a.unit_t[u_cur[warp]], t_grp[warp]);
-        atomicMax(&a.unit_t[a.K + u_cur[warp]], t_end);
-      }
+    if (lane == 0 && more && a.unit_sched != SPH_SCHED_GLOBAL) {   // the unit's first start and last end
+      unsigned long long t_end;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t_end));
+      atomicMin(&a.unit_t[u_cur[warp]], t_grp[warp]);
+      atomicMax(&a.unit_t[a.K + u_cur[warp]], t_end);
+    }
+  }
+  {
+    const unsigned long long f = warp_total(tf), c = warp_total(tc), x = warp_total(te);
+    if (lane == 0 && (f | c | x)) {                 // (a warp without a group has nothing to add)
+      atomicAdd(&a.counters[0], f);
+      atomicAdd(&a.counters[1], c);
+      atomicAdd(&a.counters[2], x);
     }
   }
   if constexpr (EXTRA) {                            // the block's adjacency bits into adj_bits
