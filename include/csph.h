@@ -65,7 +65,7 @@ extern "C" {
                                   kernel spends on unit k's particles (timing-dependent, so the
                                   rebalancing is not reproducible bit for bit) */
 
-#define SPH_SCHED_GLOBAL 0       /* list kernel: warps take groups of 32 slots (cell order) from one global
+#define SPH_SCHED_GLOBAL 0       /* list kernel: warps take groups of 8 to 32 slots (cell order) from one global
                                     counter, whatever their units */
 #define SPH_SCHED_UNITS 1        /* the Voronoi units are the work partition (Secs. 3-4 recast on one GPU):
                                     at each list build the slots are ordered unit-major (cell order

@@ -16,7 +16,6 @@ namespace csph {
 
 constexpr int kBlock = 256;          // threads of the per-particle kernels
 constexpr int kPairBlock = 128;      // threads of the pair kernel
-constexpr int kListCap = 128;        // per-particle neighbour list capacity of the pair kernel (shared memory)
 constexpr double kCellMargin = 1.0 + 0x1p-20;  // relative safety margin of D^c
 
 // Per-instance cell mesh of eq. (Dcell) on the dense grid.
@@ -496,7 +495,7 @@ cudaError_t launch_pair(sph_handle* h, const sph_state& s, cudaStream_t st);
 cudaError_t launch_pair_vjp(sph_handle* h, const sph_state& s, const void* G, const void* GR2, double* out,
                             cudaStream_t st, const void* A64 = nullptr, const void* B64 = nullptr,
                             const void* C64 = nullptr);
-// Verlet lists: build (k_pair over the (1 + beta) radius, returns at once unless vflag[0]) and
+// Verlet lists: build (k_list_build, over the (1 + beta) radius; returns at once unless vflag[0]) and
 // the pair evaluation over the lists; both only after a launch_pack in the same step, which
 // zeroes their counters
 cudaError_t launch_list_build(sph_handle* h, const sph_state& s, cudaStream_t st);

@@ -22,7 +22,7 @@ namespace {
 // are cheaper than compacting the accepted ones first.  Each lane's Kahan
 // sum takes about a quarter of the slot's pairs; the slot's four sums are
 // combined by a fixed butterfly, and the FP64 scaling of the rates is done
-// for the 32 slots of the group at once, one slot per lane.  Offsets stay
+// for up to 32 slots at once, one slot per lane.  Offsets stay
 // relative to the cells of the build and each pair's shift comes from its
 // neighbour-cell code, so the momentum fluxes stay antisymmetric bit for bit; every
 // order is fixed, so results are reproducible bit for bit.
@@ -32,7 +32,7 @@ namespace {
 // position and velocity operands are one 32-byte record read by one load (660 ->
 // 636 us at 1.125M against two arrays).  FP64: the FP64 pipe; the FP32 test runs
 // first over a segment of entries, the accepted ones are compacted and their
-// fluxes evaluated with full lanes (65k ejecta cloud, two steps, 2453 -> 1694 us).
+// fluxes evaluated with full lanes (65k ejecta cloud, two steps, 2453 -> 1694 us; today 1609).
 
 // Lanes per slot of k_pair_lists (a divisor of 32): measured on the 1.125M
 // plate impact, 16 / 8 / 4 / 2 lanes per slot take 0.89 / 0.81 / 0.75 / 0.76 ms.
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kPairBlock, MIXED ? 7 : 4) k_pair_lists(PairAr
     }
     int unit_run = -1;
     unsigned unit_load = 0;
-    // Half h of the warp takes slots g0 + 2q + h, q = 0..15.  The list reads
+    // Lanes 4 s to 4 s + 3 (half = s) take slots g0 + 8 q + s, q = 0, 1, ...  The list reads
     // are software-pipelined: the next chunk of entries (and, across slots,
     // the next slot's first chunk and count) is requested before the current
     // one is evaluated, so the DRAM latency of the lists overlaps the L2
@@ -533,15 +533,14 @@ cudaError_t launch_lists_one(const PairArgs& args_in, int blocks_per_sm, cudaStr
   const auto [sms, per_sm] = resident_blocks<k_pair_lists<MIXED, DIM, HLL, EXTRA, STAGE, KERN>>(kPairBlock);
   const int b = (blocks_per_sm > 0 && blocks_per_sm < per_sm) ? blocks_per_sm : per_sm;
   int grid = sms * b;
-  // Groups of 32 slots share the set-up and the FP64 rate formation best (a
-  // group of 8 costs ~20 % more per slot on a full chip), but a launch ends when
-  // its last groups do.  Up to 27 slots per resident warp every group would be
+  // Groups of 32 slots share the set-up best, but a launch ends when its last
+  // groups do.  Up to 27 slots per resident warp every group would be
   // the last one of its warp: groups of 8 (one pass of the warp, four lanes per
   // slot), above 16 slots per warp those go out last, after groups of 16.
   // Beyond, the last 16 slots per warp go out in groups of 8 unless a last wave
   // of 32 would be full anyway (by 5/6).  List kernel against 32 throughout,
-  // 4256 warps, no units: 9k 82 -> 33 us, 32k 88 -> 44, 77k 98 -> 71, 140k 125 ->
-  // 107, 203k 159 -> 143, 387k 256 -> 246, 874k 539 -> 530, 1.125M 677 -> 671.
+  // 4256 warps, lattices without units: 8k 91 -> 34 us, 33k 99 -> 42, 85k 105 ->
+  // 75, 185k 168 -> 135, 275k 206 -> 194, 729k 493 -> 478, 1.125M 735 -> 727.
   PairArgs args = args_in;
   const int64_t warps = (int64_t)kWarps * grid, n = args.n;
   args.big = n > 27 * warps ? 32 : 16;

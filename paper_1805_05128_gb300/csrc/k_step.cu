@@ -116,7 +116,7 @@ __device__ void block_reduce(Red& r, int dim, bool verlet) {
   }
 }
 
-// Block minimum of the dt keys only (a step's k_derive); result in thread 0.
+// Block minimum of the dt keys (k_cfl, k_kick2); result in thread 0.
 __device__ long long block_min_key(long long k) {
   __shared__ long long sh[kBlock / 32];
   k = warp_min(k);
@@ -134,8 +134,7 @@ __device__ __forceinline__ void write_part(BlockPart* part, const Red& r) {
 
 // ---------------------------------------------------------------------------
 // d, P, c and the bounding box of the current state (a mesh build outside the
-// step follows), or a step's CFL bound dt_i = eta d_i / (c_i + |v_i|)
-// (cfl_key), min-reduced into the instance's dt_key.
+// step follows).
 // ---------------------------------------------------------------------------
 __global__ void k_derive(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
                          const int64_t* __restrict__ blk_end, BlockPart* part) {
@@ -161,6 +160,8 @@ __global__ void k_derive(DevParams P, sph_state s, const int64_t* __restrict__ b
   if (threadIdx.x == 0) write_part(part, r);
 }
 
+// A step's CFL bound dt_i = eta d_i / (c_i + |v_i|) (cfl_key), min-reduced into
+// the instance's dt_key.
 __global__ void k_cfl(DevParams P, sph_state s, const int64_t* __restrict__ blk_start,
                       const int64_t* __restrict__ blk_end, const int32_t* __restrict__ blk_inst, long long* dt_key) {
   chain_entry();

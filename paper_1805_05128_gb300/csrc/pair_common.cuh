@@ -124,7 +124,7 @@ struct Ops<true> {
 // with one 32-byte load, whose four-lane passes read one run of neighbours
 // each.  As two arrays they were two gathers of 16 bytes, a quarter of the L1
 // data-pipe wavefronts of the list kernel each (88 % of that pipe's peak): list
-// kernel at 1.125M 672 -> 640 us, 387k search 1.94 -> 1.89 ms per 3 steps.
+// kernel at 1.125M 660 -> 636 us, 387k search 1.94 -> 1.88 ms per 3 steps.
 __device__ __forceinline__ void load_AB(const void* A, const void*, uint32_t j, float4& a, float4& b) {
   const float4* p = reinterpret_cast<const float4*>(A) + 2 * (size_t)j;
   asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -402,23 +402,6 @@ struct Pair {
   using V4 = typename Ops<MIXED>::V4;
   using V2 = typename Ops<MIXED>::V2;
   using VC = typename Ops<MIXED>::VC;
-
-  // Canonical separation lo -> hi.  sh: shift from i's cell to j's cell (mixed only).
-  static __device__ __forceinline__ void sep(bool ilo, const V4& Ai, const V4& Aj, T sx, T sy, T sz, T& dx,
-                                             T& dy, T& dz) {
-    const V4& lo = ilo ? Ai : Aj;
-    const V4& hi = ilo ? Aj : Ai;
-    if (MIXED) {
-      T s0 = ilo ? sx : -sx, s1 = ilo ? sy : -sy, s2 = ilo ? sz : -sz;
-      dx = (hi.x + s0) - lo.x;
-      dy = DIM >= 2 ? (hi.y + s1) - lo.y : T(0);
-      dz = DIM >= 3 ? (hi.z + s2) - lo.z : T(0);
-    } else {
-      dx = __dsub_rn(hi.x, lo.x);
-      dy = DIM >= 2 ? __dsub_rn(hi.y, lo.y) : 0.0;
-      dz = DIM >= 3 ? __dsub_rn(hi.z, lo.z) : 0.0;
-    }
-  }
 
   static __device__ __forceinline__ T r2_of(T dx, T dy, T dz) {
     if (MIXED) {
