@@ -27,7 +27,7 @@ namespace {
 // neighbour-cell code, so the momentum fluxes stay antisymmetric bit for bit; every
 // order is fixed, so results are reproducible bit for bit.
 //
-// Bound, mixed: the L1 data pipe (86 % of its cycles) and issue (76 %) together:
+// Bound, mixed: the L1 data pipe (88 % of its cycles) and issue (76 %) together:
 // an operand gather touches ~13 line quarters per 32 entries.  A neighbour's
 // position and velocity operands are one 32-byte record read by one load (660 ->
 // 636 us at 1.125M against two arrays).  FP64: the FP64 pipe; the FP32 test runs
